@@ -214,12 +214,13 @@ rewl_status configure(rewl_batch_s *b, const Config &c) {
         tab[(size_t)i].M = h->M;
         tab[(size_t)i].S = h->S;
         tab[(size_t)i].lay = rewl::fast_layout(h->M, c.lanes, c.lanes == 1);
+        const int bits = rewl::sweep_bits(h->M, c.lanes, c.lanes == 1);
         int cls = -1;
         for (size_t k = 0; k < b->classes.size(); ++k)
-            if (b->classes[k].bits == h->M.bits) cls = (int)k;
+            if (b->classes[k].bits == bits) cls = (int)k;
         if (cls < 0) {
             SweepClass sc;
-            sc.bits = h->M.bits;
+            sc.bits = bits;
             sc.lanes = c.lanes;
             b->classes.push_back(sc);
             cls = (int)b->classes.size() - 1;

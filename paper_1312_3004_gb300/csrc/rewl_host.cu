@@ -312,6 +312,10 @@ rewl_status prepare_instance(rewl_s *h, const rewl_params &p, int spin_bits, int
     M.wpc = (M.N * M.bits + 31) / 32;
     M.key0 = (uint32_t)(p.seed & 0xffffffffull);
     M.key1 = (uint32_t)(p.seed >> 32);
+    for (uint32_t r = 0; r < 10; ++r) {
+        M.rk[2 * r] = M.key0 + r * 0x9E3779B9u;
+        M.rk[2 * r + 1] = M.key1 + r * 0xBB67AE85u;
+    }
     M.divL = (uint32_t)((0x100000000ull + (unsigned long long)p.L - 1) / (unsigned long long)p.L);
     M.K = p.exchange_interval;
     M.lnf_final = p.lnf_final;

@@ -59,6 +59,7 @@ struct Model {
     int bits;                 // 4 or 8 bits per stored spin
     int wpc;                  // 32-bit words per configuration buffer
     uint32_t key0, key1;      // Philox key = seed
+    uint32_t rk[20];          // Philox round keys: key0 + r Weyl0, key1 + r Weyl1 for r = 0 .. 9
     uint32_t divL;            // ceil(2^32 / L) for site -> (x, y)
     long long K;              // WL steps per walker between exchanges
     double lnf_final, flatness;
@@ -119,7 +120,8 @@ enum : int { SWEEP_REFERENCE = 0, SWEEP_FAST = 1 };
 struct Layout {
     int stride;                 // bytes per walker (multiple of 16)
     int off_lgf, off_lat;       // byte offsets: ln g shadow (with sentinels), lattice
-    int off_q, off_e, off_bm;   // serial-loop staging and conflict marks (lane groups)
+    int off_pk, off_tab, off_bm;  // proposals, steps by bin and conflict marks of a batch (lane groups)
+    int marks;                  // entries of the conflict marks (a power of two)
 };
 
 // One instance of a batch, as the batched kernels see it.
@@ -174,6 +176,9 @@ size_t fast_smem_per_walker(const Model &M, int lanes, bool lat_global = false);
 cudaError_t launch_sweep_fast(const Model &M, const State &S, const SweepPlan &p, cudaStream_t s, bool prepare);
 
 Layout fast_layout(const Model &M, int lanes, bool lat_global = false);
+// Bits per spin while the sweep runs (lattices staged in shared memory are
+// mostly held as bytes): the kernel variant that runs the walkers of M.
+int sweep_bits(const Model &M, int lanes, bool lat_global = false);
 // A lattice above this many bytes stays in global memory in the fast sweep.
 constexpr int kSharedLatticeMax = 16384;
 // Sentinel bins beyond each end of a window in the ln g shadow.

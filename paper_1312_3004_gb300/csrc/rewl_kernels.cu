@@ -650,11 +650,12 @@ SweepPlan plan_sweep(const Model &M, int num_sms, size_t smem_optin, int kind, i
         // the rate); a thread per walker, state in global memory, once there are
         // enough of them to fill the SMs by themselves (measured crossover on
         // GB300: between 4096 and 16384 walkers)
-        // (tiny lattices: 32 proposals of a batch touch each other's neighbourhoods
-        // so often that 8-lane trees win -- measured on the L = 8 Ising workload:
-        // 2.13e7 flips/s with 8 lanes against 1.74e7 with 32)
+        // (lane groups are 32 lanes at every lattice size: a batch of 32 takes about
+        // as long as one of 8, also where the proposals of a batch touch each other
+        // -- L = 8 Ising, 8 walkers: 615 us a round of 10^4 steps against 1346 with
+        // 8 lanes and 934 with 16; q = 10, L = 20: 708 against 1415 and 1095)
         const bool chosen = lanes <= 0;
-        if (chosen) lanes = M.G <= 80 * num_sms ? (M.N <= 128 ? 8 : 32) : 1;
+        if (chosen) lanes = M.G <= 80 * num_sms ? 32 : 1;
         // a window too wide for a lane group's shared memory (its ln g shadow):
         // a thread per walker with the whole state in global memory
         if (chosen && lanes > 1 && lat_mode != 2 &&

@@ -175,11 +175,12 @@ rewl_status rebuild_tables(rewl_server_s *s) {
         d.lay = rewl::fast_layout(h->M, 32);
         tab.push_back(d);
         for (int w = 0; w < h->M.h; ++w) wins.push_back({(int)i, w});
-        auto &c = s->cls[h->M.bits == 8 ? 1 : 0];
+        auto &c = s->cls[rewl::sweep_bits(h->M, 32) == 8 ? 1 : 0];
+        auto &cw = s->cls[h->M.bits == 8 ? 1 : 0];
         int P = (int)((size_t)s->optin / (size_t)d.lay.stride);
         P = std::max(1, std::min(P, 8));
         for (int g0 = 0; g0 < h->M.G; g0 += P) c.items.push_back({(int)i, g0, std::min(P, h->M.G - g0), 0});
-        for (int g = 0; g < h->M.G; ++g) c.walkers.push_back({(int)i, g});
+        for (int g = 0; g < h->M.G; ++g) cw.walkers.push_back({(int)i, g});
         c.smem = std::max(c.smem, (size_t)P * (size_t)d.lay.stride);
         c.threads = std::max(c.threads, P * 32);
     }
@@ -219,12 +220,13 @@ rewl_status rebuild_tables(rewl_server_s *s) {
     for (int k = 0; k < 2; ++k) {
         auto &c = s->cls[k];
         c.bits = k == 1 ? 8 : 4;
+        c.wgrid = (int)((c.walkers.size() + kWalkerThreads - 1) / kWalkerThreads);
+        if (!c.walkers.empty())
+            SRV_CUDA(cudaMemcpyAsync(c.d_walkers, c.walkers.data(), c.walkers.size() * sizeof(rewl::WalkerItem),
+                                     cudaMemcpyHostToDevice, s->stream));
         if (c.items.empty()) continue;
         SRV_CUDA(cudaMemcpyAsync(c.d_items, c.items.data(), c.items.size() * sizeof(rewl::SweepItem),
                                  cudaMemcpyHostToDevice, s->stream));
-        SRV_CUDA(cudaMemcpyAsync(c.d_walkers, c.walkers.data(), c.walkers.size() * sizeof(rewl::WalkerItem),
-                                 cudaMemcpyHostToDevice, s->stream));
-        c.wgrid = (int)((c.walkers.size() + kWalkerThreads - 1) / kWalkerThreads);
         SRV_CUDA(rewl::launch_batch_sweep(c.bits, 32, nullptr, nullptr, 0, nullptr, 0, c.threads, c.smem, nullptr, true));
         const int per_sm = std::max(1, rewl::batch_sweep_ctas_per_sm(c.bits, 32, c.threads, c.smem));
         c.grid = std::min((int)c.items.size(), per_sm * s->sms);
@@ -238,7 +240,7 @@ rewl_status enqueue_round(rewl_server_s *s) {
     SRV_CUDA(cudaMemsetAsync(s->d_queues, 0, 2 * sizeof(unsigned int), s->stream));
     for (int k = 0; k < 2; ++k) {
         auto &c = s->cls[k];
-        if (c.items.empty()) continue;
+        if (s->lanes == 1 ? c.walkers.empty() : c.items.empty()) continue;
         if (s->lanes == 1)
             SRV_CUDA(rewl::launch_batch_walkers(c.bits, s->d_inst, c.d_walkers, (int)c.walkers.size(), c.wgrid,
                                                 kWalkerThreads, s->stream, false));

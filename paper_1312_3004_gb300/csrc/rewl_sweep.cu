@@ -4,28 +4,25 @@
 // bit, organised for a GPU whose FP64 pipe is narrow and slow (GB300: one DADD
 // has ~64 cycles of latency and ~2 per clock per SM of throughput):
 //
-//  * A group of S lanes (S = 1 .. 32, a power of two) owns one walker.  Each
+//  * A group of S lanes (S = 2 .. 32, a power of two) owns one walker.  Each
 //    lane prepares one of the next S proposals in parallel: Philox block,
 //    site, new value, energy change against the lattice at the start of the
-//    batch, and an integer acceptance bracket.  Proposals whose neighbourhood
-//    another proposal of the batch touches are flagged.
+//    batch, and an integer acceptance bracket.
 //  * Tagged fixed-point shadow of ln g: for the launch, every ln g value v of
 //    the walker is also held as F(v) = 2 floor(v / u) + (1 if the floor
 //    dropped bits), u = 2^(e_w - 1075), e_w seven binades below the largest
-//    value the launch can reach.  D = F(ln g(E')) - F(ln g(E)) is within three
-//    half-units of the true difference, and the reference test
-//    "u_rnd < exp(ln g(E) - ln g(E'))" is decided by D < T_lo (accept) or
-//    D >= T_hi (reject), with [T_lo, T_hi) bracketing -ln(u_rnd) with a proven
-//    margin.  Only D inside the bracket (about 1e-6 of the decisions) takes
-//    the binary64 path exp(a - b) -- the operation the reference does.
+//    value the launch can reach.  The reference test
+//    "u_rnd < exp(ln g(E) - ln g(E'))" is decided by D = F(ln g(E')) -
+//    F(ln g(E)): D < T_lo (accept) or D >= T_hi (reject), with [T_lo, T_hi)
+//    bracketing -ln(u_rnd) with a proven margin.  Only D inside the bracket
+//    (about 1e-5 of the decisions) takes the binary64 path exp(a - b) -- the
+//    operation the reference does.
 //  * ln g(E) += ln f is an integer add on the shadow (ln f = 2^-k is a whole
-//    number of half-units), rounded to 53 bits in integers when it enters the
-//    next binade; values whose shadow dropped bits take binary64 steps.
-//  * The group resolves the proposals of a batch by a tree of speculative
-//    steps: lane j decides node j of the binary tree of the next log2(S)
-//    steps from the state at the start of the window, and ballots follow the
-//    true path.  Lattice writes and the visit histogram are applied in
-//    parallel after the batch.
+//    number of half-units); a value that enters the next binade, whose shadow
+//    dropped bits, or an ln f that is no whole number takes binary64 adds.
+//  * The S proposals of a batch are resolved together, by fixed-point
+//    iteration over the whole batch (walker_sweep below).
+//  * S = 1: a thread per walker, one step after another (walker_sweep_1).
 #include <cstdint>
 
 #include "rewl_internal.cuh"
@@ -33,19 +30,30 @@
 namespace rewl {
 namespace fast {
 
-__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
-                                        uint32_t k1) {
+// Philox4x32-10 with the round keys of key word w at rk(w, r), r = 0 .. 9.
+template <typename Keys>
+__device__ __forceinline__ uint4 philox_rounds(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, Keys rk) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t a0 = c0, a2 = c2;
-        c0 = __umulhi(0xCD9E8D57u, a2) ^ c1 ^ k0;
-        c2 = __umulhi(0xD2511F53u, a0) ^ c3 ^ k1;
-        c1 = 0xCD9E8D57u * a2;
-        c3 = 0xD2511F53u * a0;
-        k0 += 0x9E3779B9u;
-        k1 += 0xBB67AE85u;
+        const unsigned long long a = 0xD2511F53ull * c0, b = 0xCD9E8D57ull * c2;  // (one wide multiply each)
+        c0 = (uint32_t)(b >> 32) ^ c1 ^ rk(0, r);
+        c2 = (uint32_t)(a >> 32) ^ c3 ^ rk(1, r);
+        c1 = (uint32_t)b;
+        c3 = (uint32_t)a;
     }
     return make_uint4(c0, c1, c2, c3);
+}
+// Lane groups: prepared round keys (constant operands: 20 wide multiplies and
+// 20 three-input logic operations a block).
+__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const uint32_t (&rk)[20]) {
+    return philox_rounds(c0, c1, c2, c3, [&](int w, int r) { return rk[2 * r + w]; });
+}
+// A thread per walker: the keys of different walkers differ, and 20 registers
+// for them would cost warps per SM.
+__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1) {
+    return philox_rounds(c0, c1, c2, c3, [&](int w, int r) {
+        return w == 0 ? k0 + (uint32_t)r * 0x9E3779B9u : k1 + (uint32_t)r * 0xBB67AE85u;
+    });
 }
 
 template <int BITS>
@@ -53,16 +61,6 @@ __device__ __forceinline__ int spin_get(const uint32_t *w, int s) {
     if (BITS == 8) return reinterpret_cast<const uint8_t *>(w)[s];
     return (int)((w[s >> 3] >> ((s & 7) << 2)) & 15u);
 }
-template <int BITS>
-__device__ __forceinline__ void spin_set(uint32_t *w, int s, int v) {
-    if (BITS == 8) {
-        reinterpret_cast<uint8_t *>(w)[s] = (uint8_t)v;
-    } else {
-        const uint32_t sh = (uint32_t)(s & 7) << 2;
-        w[s >> 3] = (w[s >> 3] & ~(15u << sh)) | ((uint32_t)v << sh);
-    }
-}
-
 struct Site4 { int r, l, d, u; };
 __device__ __forceinline__ Site4 nbrs(int s, int L, int N, uint32_t divL) {
     const int y = (int)__umulhi((uint32_t)s, divL);
@@ -73,14 +71,6 @@ __device__ __forceinline__ Site4 nbrs(int s, int L, int N, uint32_t divL) {
     n.d = (y == L - 1) ? s - (N - L) : s + L;
     n.u = (y == 0) ? s + (N - L) : s - L;
     return n;
-}
-
-template <int BITS>
-__device__ __forceinline__ int energy_change(const uint32_t *lat, const Site4 &n, int cur, int nw) {
-    const int a = spin_get<BITS>(lat, n.r), b = spin_get<BITS>(lat, n.l);
-    const int c = spin_get<BITS>(lat, n.d), d = spin_get<BITS>(lat, n.u);
-    return (int)(a == cur) + (int)(b == cur) + (int)(c == cur) + (int)(d == cur) - (int)(a == nw) -
-           (int)(b == nw) - (int)(c == nw) - (int)(d == nw);
 }
 
 // 53-bit integer of the uniform u = U * 2^-53 (27 bits of hi, 26 of lo).
@@ -114,7 +104,8 @@ __device__ __forceinline__ long long scaled_ceil(float x, int k) {
 
 // Bracket of T = -ln(u) / unit, unit = 2^-k: accept for sure if D < t_lo,
 // reject for sure if D >= t_hi, where D is within three units of the true
-// difference (the shadow's floors and inexact tags, see shadow_of).  uf = u with relative error <= 2^-23 (24 + 24 bits, one
+// difference (the shadow's floors and inexact tags, see shadow_of); a lane
+// group widens it by kSlack for the roundings inside a batch.  uf = u with relative error <= 2^-23 (24 + 24 bits, one
 // rounding; top >= 1 makes the 5 dropped bits <= 2^-24 relative); logf is
 // within 1 ulp; so |Lf - (-ln u)| <= (Lf + 1) 2^-22.9, and the margin
 // (Lf + 1) 2^-18 leaves a factor > 8 for that, for exp's own error (1 ulp of
@@ -215,19 +206,23 @@ __device__ __forceinline__ unsigned group_mask() {
 
 // Per-walker scratch of the lane group in shared memory (S > 1 only).
 struct Stage {
-    longlong2 *q;  // [S + kStagePad] bracket of proposal k as the serial loop reads it: (t_lo, t_hi - t_lo)
-    int *e;        // [S + kStagePad] energy change of proposal k as a byte step over the ln g shadow (8 dE)
-    uint32_t *bm;    // [2 nbw] marks of the sites proposed in this batch; then of those proposed twice
-    int nbw;         // ceil(min(N, kMarkBits) / 32)
-    uint32_t mmask;  // site -> mark: all bits when N <= kMarkBits, else kMarkBits - 1 (shared marks
-                     // only ever flag more proposals, never fewer)
+    uint32_t *pk;    // [S] proposal k as conflicting lanes read it: site | new value << 20
+    uint32_t *tab;   // [8 S] steps of the batch that end in bin x, at x mod 8 S; zero between uses
+    uint32_t *bm;    // [marks] lanes of the batch that propose a site, at site & mmask; zero between uses
+    uint32_t mmask;  // entries - 1 (sites share entries where N is larger: that costs comparisons only)
 };
-constexpr int kStagePad = 8;
-constexpr int kMarkBits = 8192;
-
-// A bracket no difference passes: the serial loop hands the proposal to the
-// exact step (t_lo below every in-window D, width covering every D).
-constexpr long long kForceLo = -(1LL << 62);
+// Entries of the conflict marks: the power of two at or above N, at most this.
+constexpr int kMarks = 1024;
+inline int mark_entries(int N) {
+    int e = 32;
+    while (e < N && e < kMarks) e <<= 1;
+    return e;
+}
+// Half-units by which D in a batch can miss the true difference beyond the
+// floors of shadow_of: up to 32 adds on either bin, each rounded by at most
+// half a last place (2^8 half-units for values below 2^61 units) and, for an
+// ln f that is no whole number of units, known to 2 half-units.
+constexpr long long kSlack = 1LL << 15;
 
 struct Tally {
     TieRec tie;
@@ -268,12 +263,6 @@ __device__ __forceinline__ long long lds64(uint32_t a) {
 }
 __device__ __forceinline__ void sts64(uint32_t a, long long v) {
     *reinterpret_cast<long long *>(__cvta_shared_to_generic(a)) = v;
-}
-
-template <int S, typename T>
-__device__ __forceinline__ T from_lane(unsigned gm, T x, int k) {
-    if (S == 1) return x;
-    return __shfl_sync(gm, x, k, S);
 }
 
 // One lane per walker: the steps one after another, each proposal drawn (and
@@ -398,20 +387,79 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
     E_io = Eo + lo;
 }
 
+// The exact binary64 value of a bin after `count` more ln f steps of the batch:
+// its bits before the batch (kept in lgb when the shadow F dropped bits), then
+// the reference's adds one by one.
+__device__ __noinline__ long long exact_steps(long long F, const long long *lgb, int b, int ew, double lnf, int count) {
+    double a = __longlong_as_double((F & 1) ? lgb[b] : from_units(F >> 1, ew));
+    for (int i = 0; i < count; ++i) a = __dadd_rn(a, lnf);
+    return __double_as_longlong(a);
+}
+
+// S > 1 lanes per walker: batches of S steps, lane j owning step j.
+//
+// A step's outcome depends on the earlier steps of its batch only through the
+// bin they have led to, the ln f steps they have added to the two bins it
+// compares, and the spins they have flipped around its site.  So every lane
+// evaluates its step under the present decisions of the lanes before it, all
+// at once, and the evaluations are repeated until no decision changes.  Such a
+// fixed point is unique and is the serial result: step 0 depends on nothing,
+// and if steps 0 .. j - 1 agree with the serial run, so does step j.  Each
+// evaluation makes at least one more leading step final, so at most S + 1 are
+// needed; the decisions depend on each other weakly, and the measured number
+// per batch of 32 is 1.0 .. 1.7 at a late ln f and 2 .. 7 at ln f = 1,
+// confirming evaluation included.
+//
+// What bounds it: the latency of one dependent chain per walker (with 7 walkers
+// per SM nothing else is near its limit), so every part is chosen for its
+// latency.  Measured on GB300, in cycles with their use: popcount 24 (four of
+// them 56), ballot 17, match 38, shared load 34, store-then-load 42,
+// atomic-then-load 99, leading-zero count 27, a branch on a vote about 45.
+// Hence matches and plain stores instead of shared atomics, and one branch per
+// evaluation.  q = 10, L = 80, 1024 walkers, 10^4 steps each: 1.17 -> 0.72 ms a
+// round in the first rounds (ln f = 1) and 1.10 -> 0.55 ms at ln f = 2^-20,
+// against the step trees that were here before (the decisions of the next five
+// steps at a time, 275 cycles a step).
+//
+//  * The bin before step j: the batch's start plus the accepted energy changes
+//    of the lanes before it; from four ballots (the bit planes of the changes,
+//    two's complement) and popcounts instead of a five-step shuffle scan.
+//  * ln f steps added inside the batch: at a large ln f every evaluation counts
+//    them, otherwise only when one of the at most j that precede step j could
+//    decide.  The steps before j that ended in a bin are the lanes 1 .. j that
+//    start from it: for the old bin a match of the lanes' bins, for the new one
+//    that match read through a table by bin (mod 8 S: the path spans at most
+//    4 S + 4 bins either way).
+//  * Flips: every lane leaves the lanes that propose its site at the site's
+//    entry of a table and reads the entries of its four neighbours; the energy
+//    change of a lane that others touch is recomputed from the spins at the
+//    start of the batch and the flips of the accepted touching lanes, in order,
+//    whenever those change.
+//  * A draw inside its bracket is settled when everything before it is final:
+//    the reference's binary64 test on the exact values, then the lane keeps
+//    that decision.
+//  * Commit: one add of count x ln f per distinct bin (binary64 adds one by one
+//    where the integer add is not exact), one histogram add per distinct bin,
+//    one store per flipped site.
 template <int BITS, int S>
-__device__ void walker_sweep(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb,
-                             long long *lgf, uint32_t *__restrict__ hg, const Stage &st, int g, int lo,
-                             double lnf, int &E_io, unsigned long long &t_io, Tally &tally) {
+__device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb,
+                                             long long *lgf, uint32_t *__restrict__ hg, const Stage &st, int g, int lo,
+                                             double lnf, int &E_io, unsigned long long &t_io, Tally &tally) {
     if constexpr (S == 1) {
         walker_sweep_1<BITS>(M, lat, lgb, lgf, hg, g, lo, lnf, E_io, t_io, tally);
         return;
-    }
+    } else {
     const int j = (int)(threadIdx.x & (unsigned)(S - 1));
     const unsigned gm = group_mask<S>();
+    const unsigned gbase = S == 32 ? 0u : threadIdx.x & 31u & ~(unsigned)(S - 1);
+    const unsigned bit = 1u << j, lt = bit - 1u, le = lt | bit;  // lane j; the lanes before it; both
+    const unsigned le1 = le & ~1u;  // (the bins before steps 1 .. j are those after steps 0 .. j - 1)
     const int N = M.N, L = M.L;
     constexpr int per = 32 / BITS;  // sites per lattice word
     const uint32_t qm1 = (uint32_t)(M.q - 1);
     const long long LNF = __double_as_longlong(lnf);
+    auto ballot = [&](bool p) { return __ballot_sync(gm, p) >> gbase; };
+    auto match = [&](uint32_t x) { return __match_any_sync(gm, x) >> gbase; };  // lanes with the same x
 
     // ---- fixed-point frame of this launch --------------------------------------
     long long vmax = 0;
@@ -431,328 +479,327 @@ __device__ void walker_sweep(const Model &M, uint32_t *__restrict__ lat, long lo
     }
     bool addF;
     const long long incU = exact_units(LNF, ew, addF);
-    const long long incF = incU << 1;  // ln f in half-units
+    // ln f in half-units (rounded down to whole units where it is none)
+    const unsigned long long incF = (unsigned long long)(addF ? incU << 1 : shadow_of(LNF, ew) & ~1LL);
     // every integer step inside a binade is exact when ln f is a multiple of the
     // largest last place (2^8 units for values below 2^61 units)
     const bool int_add = addF && (incU & 255) == 0;
-    if (S > 1) __syncwarp(gm);
+    // Decisions are first taken on the leading 32-bit words of the shadows, in
+    // units of 2^(32 - k); where those cannot decide, on all 64 bits (see
+    // `bracket` below).  small_k: the draws' 2^-26 fits that unit.
+    const bool small_k = __all_sync(gm, k >= 26 && k <= 57);
+    const int tsh = 58 - k;
+    // At a large ln f nearly every evaluation has to count the batch's own ln f
+    // steps: it does so at once, in whole leading words.
+    const bool heavy = __all_sync(gm, small_k && lnf >= 0x1p-7 && (uint32_t)incF == 0u);
+    const int incH = (int)(incF >> 32);
+    // ln f steps that can precede step j, in leading words (rounded up)
+    const uint32_t kinc = heavy || !small_k ? 0u : (uint32_t)((incF * (unsigned)j + 0xffffffffull) >> 32);
+    __syncwarp(gm);
 
-    // The current bin: Eo its index in the window, AF its shadow (always equal
-    // to lgf[Eo]), pcur the shared address of lgf[Eo].  A shadow >= 2^52 is the
-    // value exactly; below that the exact binary64 bits are kept in lgb.
-    int Eo = E_io - lo;
-    // (lane groups: the shadow is in shared memory; one lane: shared or global)
-    const uint32_t pbase = S > 1 ? (uint32_t)__cvta_generic_to_shared(lgf) : 0u;
-    long long AF = lgf[Eo];
-    unsigned int nacc = 0;
-    // node of this lane in the step tree (lane S - 1 has none)
-    constexpr int DP = S >= 32 ? 5 : S >= 16 ? 4 : S >= 8 ? 3 : S >= 4 ? 2 : 1;
-    const int lvl = 31 - __clz(j + 1), pre = j + 1 - (1 << lvl);
-    const unsigned lane = threadIdx.x & 31u, gbase = lane & ~(unsigned)(S - 1);
-    // its ancestors, (l, pre mod 2^l) at node index 2^l - 1 + (pre mod 2^l): which
-    // they are, and the decision each must take for the path to lead here
-    unsigned anc_mask = 0u, anc_bits = 0u;
-    bool tl[DP > 1 ? DP - 1 : 1], tb[DP > 1 ? DP - 1 : 1];  // step l on the path; taken as a move
-#pragma unroll
-    for (int l = 0; l < DP - 1; ++l) {
-        tl[l] = l < lvl;
-        tb[l] = l < lvl && ((pre >> l) & 1);
-        if (l < lvl) {
-            const int a = (1 << l) - 1 + (pre & ((1 << l) - 1));
-            anc_mask |= 1u << a;
-            anc_bits |= (unsigned)((pre >> l) & 1) << a;
+    const uint32_t pbase = (uint32_t)__cvta_generic_to_shared(lgf);
+    const uint32_t tbase = (uint32_t)__cvta_generic_to_shared(st.tab);
+    const uint32_t mbase = (uint32_t)__cvta_generic_to_shared(st.bm);
+    const int pmin = (int)pbase - (kPad - 4) * 8, pmax = (int)pbase + (M.B + kPad - 5) * 8;
+    uint32_t pcur = pbase + (uint32_t)(E_io - lo) * 8u;  // shared address of the current bin's shadow
+    unsigned int nacc = 0, nseq = 0;
+    auto lds32 = [](uint32_t a) { return *reinterpret_cast<const uint32_t *>(__cvta_shared_to_generic(a)); };
+    auto sts32 = [](uint32_t a, uint32_t v) { *reinterpret_cast<uint32_t *>(__cvta_shared_to_generic(a)) = v; };
+    auto lead = [&](uint32_t a) { return (int)lds32(a + 4u); };  // leading word of a shadow
+    // the entry of tab that stands for the bin whose shadow is at shared address a
+    auto tab_at = [&](uint32_t a) { return tbase + ((a >> 1) & (uint32_t)(32 * S - 4)); };
+    // conflict marks: the lanes of the batch that propose a site, at the site's
+    // entry (sites share entries where N is larger than the table)
+    const uint32_t mbytes = st.mmask << 2;
+    auto mark_at = [&](int s) { return mbase + (((uint32_t)s << 2) & mbytes); };
+    const bool shared_marks = (uint32_t)N > st.mmask + 1u;
+
+    // The part of a proposal that needs no state: site, neighbours, new value,
+    // T = -ln u in 2^-26 (kTiny: u < 2^-24, only D < 0 is decided by it), the
+    // lanes that propose the same site or share its entry of the marks, and
+    // [blo, blo + bw): the leading-word differences that do not decide.  The
+    // true difference D 2^-32 lies strictly within 1 of the difference of the
+    // leading words, kSlack is far below a leading word's unit, and out of the
+    // window the difference is at least 2^30 - 2, above every T at tsh >= 1.
+    constexpr int kTiny = 0x7fffffff;
+    struct Draw {
+        int site, v, T, blo;
+        uint32_t bw;
+        unsigned same_site, same_mark;
+        Site4 nb;
+    };
+    auto random = [&](unsigned long long t) {
+        return philox((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)g, DOM_WL, M.rk);
+    };
+    auto draw = [&](unsigned long long t) {
+        const uint4 r = random(t);
+        Draw d;
+        d.site = (int)__umulhi(r.x, (uint32_t)N);
+        d.v = (int)__umulhi(r.y, qm1);
+        d.nb = nbrs(d.site, L, N, M.divL);
+        d.same_site = match((uint32_t)d.site);
+        d.same_mark = match(mark_at(d.site));
+        // as accept_bracket, in integers: u from its leading 27 bits and the rest
+        // (relative error below 2^-23), -ln u from lg2.approx (absolute or relative
+        // error at most 2^-22, times ln 2) and rounded to 2^-26: together below
+        // (Lf + 1) 2^-21; the margin is (Lf + 1) 2^-18
+        const float uf = fmaf((float)(r.z & ~31u), 0x1p-32f, (float)r.w * 0x1p-59f);
+        float l2;
+        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l2) : "f"(uf));
+        d.T = r.z < 256u ? kTiny : __float2int_rn(l2 * -0x1.62e43p+25f);  // below 2^31 for u >= 2^-24
+        const int mg = (d.T >> 18) + 260;  // (Lf + 1) 2^-18, rounded up
+        d.blo = ((d.T - mg) >> tsh) - 1;
+        d.bw = (uint32_t)(((d.T + mg) >> tsh) + 3 - d.blo);
+        if (d.T == kTiny || !small_k) {
+            d.blo = small_k ? -2 : -0x7fffffff;
+            d.bw = 0xfffffff0u;
         }
-    }
+        return d;
+    };
+    // the same bracket in half-units, from step t's draw
+    auto bracket = [&](int T, unsigned long long t, long long &blo, unsigned long long &width) {
+        long long bhi;
+        if (small_k && T != kTiny) {
+            const int mg = (T >> 18) + 260;
+            blo = (long long)(T - mg) << (k - 26);
+            bhi = (long long)(T + mg) << (k - 26);
+        } else {
+            const uint4 r = random(t);
+            accept_bracket(u53(r.z, r.w), k, blo, bhi);
+        }
+        width = (unsigned long long)(bhi - blo) + 2ull * kSlack;
+        blo -= kSlack;
+    };
+
+    Draw next = draw(t_io + (unsigned long long)j);
+    int cur0, sr0, sl0, sd0, su0;
+    auto read_spins = [&]() {
+        cur0 = spin_get<BITS>(lat, next.site);
+        sr0 = spin_get<BITS>(lat, next.nb.r);
+        sl0 = spin_get<BITS>(lat, next.nb.l);
+        sd0 = spin_get<BITS>(lat, next.nb.d);
+        su0 = spin_get<BITS>(lat, next.nb.u);
+    };
+    read_spins();
+    sts32(mark_at(next.site), next.same_mark);
+    __syncwarp(gm);
 
     for (long long base = 0; base < M.K; base += S) {
         const int n = (int)((M.K - base) < S ? (M.K - base) : S);
-        // ---- parallel phase: lane j prepares proposal t + j --------------------
-        int site = N + j, v = 0, dE = 0, word = 0;
-        Site4 nb{0, 0, 0, 0};
-        uint32_t xr = 0;  // the flip as an xor on its lattice word
-        longlong2 th = make_longlong2(0, kNoReject);
-        unsigned long long U = 0;
-        if (j < n) {
-            const unsigned long long tj = t_io + (unsigned long long)j;
-            const uint4 r = philox((uint32_t)tj, (uint32_t)(tj >> 32), (uint32_t)g, DOM_WL, M.key0, M.key1);
-            site = (int)__umulhi(r.x, (uint32_t)N);
-            v = (int)__umulhi(r.y, qm1);
-            const int cur = spin_get<BITS>(lat, site);
-            const int nw = v + (v >= cur);
-            nb = nbrs(site, L, N, M.divL);
-            dE = energy_change<BITS>(lat, nb, cur, nw);
-            word = site / per;
-            xr = (uint32_t)(cur ^ nw) << ((site & (per - 1)) * BITS);
-            U = u53(r.z, r.w);
-            accept_bracket(U, k, th.x, th.y);
+        // ---- lane j prepares proposal t + j against the lattice as it is --------
+        // (its spins were read, and its site marked, at the end of the last batch)
+        Draw d = next;
+        const int site = d.site;
+        const Site4 nb = d.nb;
+        int cur = cur0, nw = d.v + (d.v >= cur0);
+        int dE = (int)(sr0 == cur) + (int)(sl0 == cur) + (int)(sd0 == cur) + (int)(su0 == cur) - (int)(sr0 == nw) -
+                 (int)(sl0 == nw) - (int)(sd0 == nw) - (int)(su0 == nw);
+        // earlier lanes whose flip would change this proposal
+        unsigned touch = (d.same_mark | lds32(mark_at(nb.r)) | lds32(mark_at(nb.l)) | lds32(mark_at(nb.d)) |
+                          lds32(mark_at(nb.u))) & lt;
+        if (n < S && j >= n) {  // past the launch's last step: never accepted
+            d.blo = (int)0x80000000;
+            d.bw = 0u;
         }
-        bool flag = false;  // an earlier proposal of the batch may change dE
-        longlong2 q1 = make_longlong2(th.x, th.y - th.x);
-        if (S > 1) {
-            // ---- conflict marks: sites proposed in this batch -------------------
-            // (a site proposed twice marks both proposals: the later one needs it)
-            const uint32_t ms = (uint32_t)site & st.mmask;
-            const int wsite = (int)(ms >> 5);
-            const uint32_t bsite = 1u << (ms & 31);
-            uint32_t *dup = st.bm + st.nbw;
-            if (j < n && (atomicOr(&st.bm[wsite], bsite) & bsite)) atomicOr(&dup[wsite], bsite);
-            __syncwarp(gm);
-            if (j < n) {
-                const uint32_t mr = (uint32_t)nb.r & st.mmask, ml = (uint32_t)nb.l & st.mmask;
-                const uint32_t md = (uint32_t)nb.d & st.mmask, mu = (uint32_t)nb.u & st.mmask;
-                flag = ((dup[wsite] >> (ms & 31)) | (st.bm[mr >> 5] >> (mr & 31)) | (st.bm[ml >> 5] >> (ml & 31)) |
-                        (st.bm[md >> 5] >> (md & 31)) | (st.bm[mu >> 5] >> (mu & 31))) & 1u;
-                st.q[j] = flag ? make_longlong2(kForceLo, -1LL) : q1;
-                st.e[j] = dE * 8;
-            }
-            for (int p = j; p < kStagePad; p += S) {  // entries past the batch: read, never taken
-                st.q[n + p] = make_longlong2(0, 0);
-                st.e[n + p] = 0;
-            }
-            __syncwarp(gm);
-            if (j < n) {  // every marked word belongs to some lane's site
-                st.bm[wsite] = 0u;
-                dup[wsite] = 0u;
+        // with up to kinc ln f steps on either side (kTiny: already everything from -2 up)
+        const int blo2 = d.blo - (int)kinc;
+        const uint32_t bw2 = d.bw == 0xfffffff0u || d.bw == 0u ? d.bw : d.bw + 2u * kinc;
+        // first evaluation: as if every step started from the batch's first bin
+        const int D0 = lead(pcur + (uint32_t)(dE * 8)) - lead(pcur);
+        // bit planes of the energy changes (two's complement)
+        unsigned q0 = ballot(dE & 1), q1 = ballot(dE & 2), q2 = ballot(dE & 4), q3 = ballot(dE & 8);
+        unsigned A = ballot(D0 < d.blo);  // the steps that accept, as presently known
+        unsigned fl = ballot(touch != 0u);
+        // the state-free part of the next batch's proposals: independent
+        // instructions for the waits of this batch
+        next = draw(t_io + (unsigned long long)(S + j));
+        __syncwarp(gm);
+        sts32(mark_at(site), 0u);
+        if (fl) {
+            st.pk[j] = (uint32_t)site | ((uint32_t)nw << 20);
+            if (shared_marks) {  // keep the lanes that do touch
+                __syncwarp(gm);
+                unsigned real = 0u;
+                for (unsigned rest = touch; rest; rest &= rest - 1u) {
+                    const int ps = (int)(st.pk[__ffs((int)rest) - 1] & 0xfffffu);
+                    if (ps == site || ps == nb.r || ps == nb.l || ps == nb.d || ps == nb.u) real |= rest & (0u - rest);
+                }
+                touch = real;
+                fl = ballot(touch != 0u);
             }
         }
-        unsigned flagm = S > 1 ? __ballot_sync(gm, flag) >> gbase : 0u;  // the flagged steps
 
-        // ---- serial phase: the group resolves the proposals in order ------------
-        // accm: steps of the batch that accepted; done: those already written to
-        // the lattice.  The lattice and the histogram are brought up to date in
-        // parallel after the batch (and the lattice before an exact step).
-        unsigned accm = 0, done = 0;
-        const int Eb = Eo;
-        uint32_t pcur = pbase + (uint32_t)Eo * 8u;
-        int kk = 0;
-        while (kk < n) {
-            if (int_add) {
-                if constexpr (S == 1) {
-                    // ---- fast steps: integer decision and ln f step ---------------
-                    // The step is computed speculatively; a step that needs more (a
-                    // draw inside the bracket, a value with dropped bits, a binade
-                    // crossing) leaves the loop before it changes anything.
-                    const int En = Eo + dE;
-                    const long long BF = lgf[En];  // beyond the window: kOutside
-                    const long long D = BF - AF;
-                    const bool acc = D < q1.x;
-                    const bool unsure = (unsigned long long)D - (unsigned long long)q1.x < (unsigned long long)q1.y;
-                    const long long cur = acc ? BF : AF;  // with dE = 0 both are the current shadow
-                    const long long AF2 = cur + incF;
-                    const uint32_t hc = (uint32_t)((unsigned long long)cur >> 32);
-                    const uint32_t h2 = (uint32_t)((unsigned long long)AF2 >> 32);
-                    if (!(unsure || (cur & 1) || (h2 ^ hc) > hc)) {
-                        Eo = acc ? En : Eo;
-                        AF = AF2;
-                        lgf[Eo] = AF;
-                        accm |= acc ? 1u : 0u;
-                        kk = 1;
+        // ---- evaluations until nothing changes -----------------------------------
+        unsigned moved = 0u, last = 0u;
+        uint32_t pre, to;  // the bins step j compares, as addresses of their shadows
+        // energy changes under the present flips of the touching lanes, where those changed
+        auto reflip = [&]() {
+            const unsigned ta = touch & A;
+            const bool need = ta != last || (touch & moved) != 0u;
+            moved = 0u;
+            if (ballot(need)) {
+                __syncwarp(gm);
+                bool ch = false;
+                if (need) {
+                    int c = cur0, sr = sr0, sl = sl0, sd = sd0, su = su0;
+                    for (unsigned rest = ta; rest; rest &= rest - 1u) {
+                        const uint32_t pk = st.pk[__ffs((int)rest) - 1];
+                        const int ps = (int)(pk & 0xfffffu), pv = (int)(pk >> 20);
+                        c = ps == site ? pv : c;
+                        sr = ps == nb.r ? pv : sr;
+                        sl = ps == nb.l ? pv : sl;
+                        sd = ps == nb.d ? pv : sd;
+                        su = ps == nb.u ? pv : su;
                     }
-                } else {
-                    // ---- step tree: lane j decides node j of the tree of the next DP
-                    // steps (level lvl = the step, prefix pre = the decisions taken
-                    // before it on the way there), all from the state at the start of
-                    // the window; the ballots then follow the decisions from the
-                    // root.  A node whose step needs more (a proposal whose
-                    // neighbourhood may have changed, a draw inside the bracket, a
-                    // value with dropped bits, a binade crossing) ends the window
-                    // there, and the exact step below takes it.
-                    //
-                    // The path part of a window starting at step k0 needs no state.
-                    struct Prep {
-                        int m, oA, oB;
-                        int e8[DP];  // energy changes of the window's steps (byte steps)
-                        unsigned long long incA, incB;
-                        longlong2 kq;
-                    };
-                    auto prep = [&](int k0) {
-                        Prep P;
-                        P.m = min(DP, n - k0);
-                        int *e8l = P.e8;
-#pragma unroll
-                        for (int l = 0; l < DP; ++l) e8l[l] = st.e[k0 + l];
-                        const int e8i = st.e[k0 + lvl];
-                        P.kq = st.q[k0 + lvl];
-                        // bins of the path to this node, as offsets from the current one
-                        int post[DP > 1 ? DP - 1 : 1];
-                        int oA = 0;
-#pragma unroll
-                        for (int l = 0; l < DP - 1; ++l) {
-                            if (tb[l]) oA += e8l[l];
-                            post[l] = oA;  // the bin after step l (l < lvl)
-                        }
-                        P.oA = oA;
-                        P.oB = oA + e8i;
-                        // ln f steps the path has already added to the two bins
-                        int cA = 0, cB = 0;
-#pragma unroll
-                        for (int l = 0; l < DP - 1; ++l) {
-                            if (tl[l]) {
-                                cA += post[l] == P.oA ? 1 : 0;
-                                cB += post[l] == P.oB ? 1 : 0;
-                            }
-                        }
-                        P.incA = (unsigned long long)incF * (unsigned)cA;
-                        P.incB = (unsigned long long)incF * (unsigned)cB;
-                        return P;
-                    };
-                    for (;;) {
-                        const Prep P = prep(kk);
-                        const int m = P.m;
-                        const longlong2 kq = P.kq;
-                        // the node's decision (off the true path the values are
-                        // meaningless, possibly wrapped, and never used)
-                        const uint32_t pA = pcur + (uint32_t)P.oA, pB = pcur + (uint32_t)P.oB;
-                        const long long Am = lds64(pA), Bm = lds64(pB);
-                        const long long A = (long long)((unsigned long long)Am + P.incA);
-                        const long long B = (long long)((unsigned long long)Bm + P.incB);
-                        const long long D = (long long)((unsigned long long)B - (unsigned long long)A);
-                        const bool dec = D < kq.x;
-                        const bool unsure =
-                            (unsigned long long)D - (unsigned long long)kq.x < (unsigned long long)kq.y;
-                        const long long cur = dec ? B : A;
-                        const long long A2 = (long long)((unsigned long long)cur + (unsigned long long)incF);
-                        const uint32_t hc = (uint32_t)((unsigned long long)cur >> 32);
-                        const uint32_t h2 = (uint32_t)((unsigned long long)A2 >> 32);
-                        const bool act = lvl < m;
-                        const bool bad = unsure || (cur & 1) || (h2 ^ hc) > hc;
-                        const unsigned bd = __ballot_sync(gm, act && dec) >> gbase;
-                        const unsigned bb = __ballot_sync(gm, act && bad) >> gbase;
-                        // reached: every ancestor decided as the prefix says, and cleanly
-                        const bool reached = act && (((bd ^ anc_bits) | bb) & anc_mask) == 0u;
-                        const unsigned R = __ballot_sync(gm, reached) >> gbase;  // the true path
-                        const int deep = 31 - __clz((int)R);
-                        const bool dbad = (bb >> deep) & 1u;
-                        const int c = (31 - __clz(deep + 1)) + (dbad ? 0 : 1);  // steps taken
-                        const bool commit = reached && !bad;
-                        // the decisions on the true path are the deepest node's prefix
-                        const int bits = __shfl_sync(gm, (commit && dec) ? pre | (1 << lvl) : pre, deep, S);
-                        // write the ln g values of the steps taken, level by level so
-                        // that the latest value of a bin is the one that stays
-                        const uint32_t pp = dec ? pB : pA;
-#pragma unroll
-                        for (int l = 0; l < DP; ++l) {
-                            if (commit && lvl == l) sts64(pp, A2);
-                            if (l + 1 < DP) __syncwarp(gm);
-                        }
-                        pcur = __shfl_sync(gm, (bad || !dec) ? pA : pB, deep, S);
-                        AF = __shfl_sync(gm, bad ? A : A2, deep, S);
-                        __syncwarp(gm);
-                        accm |= ((unsigned)bits & ((1u << c) - 1u)) << kk;
-                        kk += c;
-                        if (c < m || kk >= n) break;
-                    }
+                    last = ta;
+                    cur = c;
+                    const int w = d.v + (d.v >= c);
+                    ch = w != nw;
+                    nw = w;
+                    dE = (int)(sr == c) + (int)(sl == c) + (int)(sd == c) + (int)(su == c) - (int)(sr == w) -
+                         (int)(sl == w) - (int)(sd == w) - (int)(su == w);
                 }
-                if constexpr (S > 1) Eo = (int)((pcur - pbase) >> 3);
-                if (kk >= n) break;
-            }
-            if (S > 1 && int_add && ((flagm >> kk) & 1u)) {
-                // ---- a proposal whose neighbourhood may have changed: its lane
-                // recomputes it against the lattice as of this step, and the
-                // windows go on from it
-                if (((accm & ~done) >> j) & 1u) atomicXor(&lat[word], xr);
-                done = accm;
                 __syncwarp(gm);
-                if (j == kk) {
-                    const int c0 = spin_get<BITS>(lat, site);
-                    const int nw0 = v + (v >= c0);
-                    dE = energy_change<BITS>(lat, nb, c0, nw0);
-                    xr = (uint32_t)(c0 ^ nw0) << ((site & (per - 1)) * BITS);
-                    flag = false;
-                    st.q[kk] = q1;
-                    st.e[kk] = dE * 8;
+                if (ch) st.pk[j] = (uint32_t)site | ((uint32_t)nw << 20);
+                moved = ballot(ch);
+                q0 = ballot(dE & 1);
+                q1 = ballot(dE & 2);
+                q2 = ballot(dE & 4);
+                q3 = ballot(dE & 8);
+            }
+        };
+        // the bins of step j under the decisions A (a wrong guess can lie outside the window)
+        auto place = [&]() {
+            const uint32_t p = pcur + 8u * __popc(q0 & A & lt) + 16u * __popc(q1 & A & lt) +
+                               32u * __popc(q2 & A & lt) - 64u * __popc(q3 & A & lt);
+            pre = (uint32_t)max(pmin, min((int)p, pmax));
+            to = pre + (uint32_t)(dE * 8);
+        };
+        // ln f steps the path adds to step j's new bin before it, less those it
+        // adds to its old one: the lanes that start from a bin, through tab
+        auto counted = [&]() {
+            const unsigned here = match(pre);
+            const uint32_t slot = tab_at(pre);
+            __syncwarp(gm);
+            sts32(slot, here);
+            __syncwarp(gm);
+            const unsigned there = lds32(tab_at(to));
+            __syncwarp(gm);
+            sts32(slot, 0u);
+            return __popc(there & le1) - __popc(here & le1);
+        };
+        int D;
+        if (heavy) {
+            for (;;) {
+                if (fl) reflip();
+                place();
+                D = lead(to) - lead(pre) + incH * counted();
+                const unsigned A2 = ballot(D < d.blo);
+                if (A2 == A && moved == 0u) break;
+                A = A2;
+            }
+        } else {
+            for (;;) {
+                if (fl) reflip();
+                place();
+                D = lead(to) - lead(pre);
+                const unsigned A2 = ballot(D < d.blo);
+                if (A2 == A && moved == 0u) break;
+                A = A2;
+            }
+        }
+        if (ballot(heavy ? (uint32_t)(D - d.blo) < d.bw : (uint32_t)(D - blo2) < bw2)) {
+            // a step the leading words do not decide: on from here with all 64 bits
+            // and the batch's own ln f steps
+            long long b64;
+            unsigned long long w64;
+            bracket(d.T, t_io + (unsigned long long)j, b64, w64);
+            unsigned fm = 0u, fv = 0u;  // steps settled in binary64, and those of them that accept
+            for (;;) {
+                if (fl) reflip();
+                place();
+                const unsigned long long D64 = (unsigned long long)lds64(to) - (unsigned long long)lds64(pre) +
+                                               incF * (unsigned long long)(long long)counted();
+                const unsigned A2 = (ballot(j < n && (long long)D64 < b64) & ~fm) | fv;
+                const unsigned um = ballot(j < n && D64 - (unsigned long long)b64 < w64) & ~fm;
+                if (A2 != A || moved != 0u) {
+                    A = A2;
+                    continue;
                 }
-                flagm &= ~(1u << kk);
+                if (um == 0u) break;
+                // the first undecided step: the reference's test in binary64
+                const int f = __ffs((int)um) - 1;
+                const unsigned here = match(pre);
                 __syncwarp(gm);
-                continue;
-            }
-            // ---- the same step, every case done exactly ---------------------------
-            if (S > 1) {  // the lattice as of this step
-                if (((accm & ~done) >> j) & 1u) atomicXor(&lat[word], xr);
-                done = accm;
+                sts32(tab_at(pre), here);
                 __syncwarp(gm);
-            }
-            const int ks = from_lane<S>(gm, site, kk);
-            int kdE = from_lane<S>(gm, dE, kk);
-            int kword = from_lane<S>(gm, word, kk);
-            uint32_t kxr = from_lane<S>(gm, xr, kk);
-            const long long tlo = from_lane<S>(gm, th.x, kk), thi = from_lane<S>(gm, th.y, kk);
-            if (S > 1 && from_lane<S>(gm, (int)flag, kk)) {  // recompute against the current lattice
-                const int kv = from_lane<S>(gm, v, kk);
-                const int kc = spin_get<BITS>(lat, ks);
-                const int knw = kv + (kv >= kc);
-                kdE = energy_change<BITS>(lat, nbrs(ks, L, N, M.divL), kc, knw);
-                kword = ks / per;
-                kxr = (uint32_t)(kc ^ knw) << ((ks & (per - 1)) * BITS);
-            }
-            const int En = Eo + kdE;
-            const long long BF = lgf[REWL_IDX(En, -kPad, M.B + kPad, tally.bad)];
-            const long long D = BF - AF;
-            bool acc = D < tlo;
-            if (!acc && D < thi) {  // inside the bracket (never beyond the window)
+                long long Ab = 0, Bb = 0;
+                if (j == f) {
+                    const int cA = __popc(here & le1), cB = __popc(lds32(tab_at(to)) & le1);
+                    Ab = exact_steps(lds64(pre), lgb, REWL_IDX((int)(pre - pbase) / 8, 0, M.B, tally.bad), ew, lnf, cA);
+                    Bb = exact_steps(lds64(to), lgb, REWL_IDX((int)(to - pbase) / 8, 0, M.B, tally.bad), ew, lnf, cB);
+                }
+                __syncwarp(gm);
+                sts32(tab_at(pre), 0u);
+                Ab = __shfl_sync(gm, Ab, f, S);
+                Bb = __shfl_sync(gm, Bb, f, S);
+                const unsigned long long tf = t_io + (unsigned long long)f;
+                const uint4 r = random(tf);
                 tally.slow += 1;
-                const unsigned long long kU = from_lane<S>(gm, U, kk);
-                const long long Ab = (AF & 1) ? lgb[REWL_IDX(Eo, 0, M.B, tally.bad)] : from_units(AF >> 1, ew);
-                const long long Bb = (BF & 1) ? lgb[REWL_IDX(En, 0, M.B, tally.bad)] : from_units(BF >> 1, ew);
-                acc = kdE == 0 ? true : exact_accept(Ab, Bb, kU, &tally.tie, t_io + (unsigned long long)kk);
+                const bool ok = ballot(exact_accept(Ab, Bb, u53(r.z, r.w), &tally.tie, tf)) != 0u;
+                fm |= 1u << f;
+                if (ok) fv |= 1u << f;
+                A = (A & ~fm) | fv;
             }
-            const long long cur = acc ? BF : AF;
-            const int Eb2 = acc ? En : Eo;
-            long long AF2 = cur + incF;
-            if (!int_add || (cur & 1)) {  // ln g(E) += ln f in binary64
-                tally.seq += 1;
-                const long long Ab = (cur & 1) ? lgb[REWL_IDX(Eb2, 0, M.B, tally.bad)] : from_units(cur >> 1, ew);
-                const long long A2 = exact_add(Ab, lnf);
-                lgb[REWL_IDX(Eb2, 0, M.B, tally.bad)] = A2;
-                AF2 = shadow_of(A2, ew);
-            } else {
-                AF2 = round_shadow(AF2);
-            }
-            Eo = Eb2;
-            AF = AF2;
-            lgf[REWL_IDX(Eo, 0, M.B, tally.bad)] = AF;
-            pcur = pbase + (uint32_t)Eo * 8u;
-            if (acc) {
-                if (S == 1 || j == 0) atomicXor(&lat[kword], kxr);
-                accm |= 1u << kk;
-            }
-            done |= accm & (1u << kk);
-            if (j == kk) dE = kdE;  // the lane's record of its step, for the histogram
-            ++kk;
         }
 
-        // ---- after the batch: lattice and histogram ----------------------------
-        // (atomics whose result is not used: the walker does not wait for them)
-        if (((accm & ~done) >> j) & 1u) atomicXor(&lat[word], xr);
-        // the bin after step j: the batch's start plus the accepted moves up to j
-        int x = (j < n && ((accm >> j) & 1u)) ? dE : 0;
-#pragma unroll
-        for (int o = 1; o < S; o <<= 1) {
-            const int y = __shfl_up_sync(gm, x, o, S);
-            if (j >= o) x += y;
+        // ---- commit ---------------------------------------------------------------
+        // the lattice, and at once the next proposals' spins and marks, whose
+        // reads run under the ln g updates
+        const bool acc = (A & bit) != 0u;
+        if (BITS == 8) {  // the site's last accepted value stays
+            if (acc && (d.same_site & A & ~le) == 0u) reinterpret_cast<uint8_t *>(lat)[site] = (uint8_t)nw;
+        } else if (acc) {
+            atomicXor(&lat[site / per], (uint32_t)(cur ^ nw) << ((site & (per - 1)) * BITS));
         }
-        const int bin = Eb + x;
-        if (S == 1) {
-            atomicAdd(&hg[REWL_IDX(bin, 0, M.B, tally.bad)], 1u);
-        } else {  // one add per run of equal bins, by the run's last step
-            const int nxt = __shfl_down_sync(gm, bin, 1, S);
-            const bool last = j < n && (j == n - 1 || nxt != bin);
-            const unsigned ends = __ballot_sync(gm, last) >> gbase;
-            const unsigned below = ends & ((1u << j) - 1u);  // j < 32
-            if (last) atomicAdd(&hg[REWL_IDX(bin, 0, M.B, tally.bad)], (uint32_t)(j - (below ? 31 - __clz((int)below) : -1)));
+        const uint32_t at = acc ? to : pre;  // the bin after the step
+        const unsigned steps = match(j < n ? at : 0u);
+        __syncwarp(gm);
+        read_spins();
+        sts32(mark_at(next.site), next.same_mark);
+        if (j < n && (steps & ~le) == 0u) {  // the bin's last step: its lane writes for all of them
+            const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad), c = __popc(steps);
+            const long long F = lds64(at);
+            long long F2 = (long long)((unsigned long long)F + incF * (unsigned)c);
+            const uint32_t h1 = (uint32_t)((unsigned long long)F >> 32), h2 = (uint32_t)((unsigned long long)F2 >> 32);
+            if (!int_add || (F & 1) || (h2 ^ h1) > h1) {  // binary64 adds
+                const long long v = exact_steps(F, lgb, b, ew, lnf, c);
+                F2 = shadow_of(v, ew);
+                if (F2 & 1) lgb[b] = v;
+                nseq += (unsigned)c;
+            }
+            sts64(at, F2);
+            atomicAdd(&hg[b], (uint32_t)c);  // (result not used: the walker does not wait)
         }
-        nacc += (uint32_t)__popc(accm);
-        if (S > 1) __syncwarp(gm);
+        pcur = __shfl_sync(gm, at, n - 1, S);
+        nacc += acc ? 1u : 0u;
         t_io += (unsigned long long)n;
+        __syncwarp(gm);
     }
-    if (S > 1) __syncwarp(gm);
     // the binary64 array from the authoritative shadow
     for (int b = j; b < M.B; b += S) {
         const long long F = lgf[b];
         if (!(F & 1)) lgb[b] = from_units(F >> 1, ew);
     }
+#pragma unroll
+    for (int o = 1; o < S; o <<= 1) {
+        nseq += __shfl_xor_sync(gm, nseq, o);
+        nacc += __shfl_xor_sync(gm, nacc, o);
+    }
+    tally.seq += nseq;
     tally.acc += nacc;
-    E_io = Eo + lo;
+    E_io = (int)(pcur - pbase) / 8 + lo;
+    }
 }
 
 // P walkers g0 .. g0 + P - 1 of one instance: stage their lattices in shared
@@ -760,36 +807,79 @@ __device__ void walker_sweep(const Model &M, uint32_t *__restrict__ lat, long lo
 // steps (one lane group per walker), write the lattices back.  The binary64
 // ln g and the histogram of each walker stay in global memory: the launch
 // reads ln g once to build the shadow and writes it back once at the end.
+// BITS is the packing while the sweep runs: 4-bit configurations are staged as
+// bytes where BITS = 8.
+template <int BITS>
+__device__ __forceinline__ void stage_lattice(const Model &M, uint32_t *lat, const uint32_t *src) {
+    if (BITS == 8 && M.bits == 4) {
+        for (int i = threadIdx.x; i < M.wpc; i += blockDim.x) {  // eight 4-bit fields to eight bytes
+            const uint32_t w = src[i];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t x = (w >> (16 * h)) & 0xffffu;
+                x = (x | (x << 8)) & 0x00ff00ffu;
+                x = (x | (x << 4)) & 0x0f0f0f0fu;
+                if (8 * i + 4 * h < M.N) lat[2 * i + h] = x;
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < M.wpc; i += blockDim.x) lat[i] = src[i];
+    }
+}
+template <int BITS>
+__device__ __forceinline__ void unstage_lattice(const Model &M, uint32_t *dst, const uint32_t *lat) {
+    if (BITS == 8 && M.bits == 4) {
+        for (int i = threadIdx.x; i < M.wpc; i += blockDim.x) {
+            uint32_t w = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t x = 8 * i + 4 * h < M.N ? lat[2 * i + h] : 0u;
+                x = (x | (x >> 4)) & 0x00ff00ffu;
+                x = (x | (x >> 8)) & 0xffffu;
+                w |= x << (16 * h);
+            }
+            dst[i] = w;
+        }
+    } else {
+        for (int i = threadIdx.x; i < M.wpc; i += blockDim.x) dst[i] = lat[i];
+    }
+}
+
 template <int BITS, int S, bool LG>
-__device__ void sweep_block(const Model &M, const State &Sg, int g0, int P, const Layout &lay, unsigned char *smem) {
-    if (*(volatile unsigned int *)&Sg.ctl->all_done) return;
-    const int nbw = (min(M.N, kMarkBits) + 31) / 32;  // conflict-mark words
+__device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int g0, int P, const Layout &lay,
+                                            unsigned char *smem) {
+    // (votes and the broadcast of the group index tell the compiler that whole
+    // warps take each branch, which spares a divergence check at every ballot)
+    if (__any_sync(0xffffffffu, *(volatile unsigned int *)&Sg.ctl->all_done)) return;
     for (int p = 0; p < P; ++p) {
         const int g = g0 + p;
         if (g >= M.G || Sg.done[g / M.m]) continue;
         unsigned char *base = smem + (size_t)p * lay.stride;
-        if (!LG) {
-            uint32_t *lat = reinterpret_cast<uint32_t *>(base + lay.off_lat);
-            const uint32_t *src_lat = Sg.spins + (size_t)Sg.slot_cfg[g] * M.wpc;
-            for (int i = threadIdx.x; i < M.wpc; i += blockDim.x) lat[i] = src_lat[i];
-        }
+        if (!LG)
+            stage_lattice<BITS>(M, reinterpret_cast<uint32_t *>(base + lay.off_lat),
+                                Sg.spins + (size_t)Sg.slot_cfg[g] * M.wpc);
         if (S > 1) {
             uint32_t *bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
-            for (int i = threadIdx.x; i < 2 * nbw; i += blockDim.x) bm[i] = 0u;
+            for (int i = threadIdx.x; i < lay.marks; i += blockDim.x) bm[i] = 0u;
+            uint32_t *tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
+            for (int i = threadIdx.x; i < 8 * S; i += blockDim.x) tab[i] = 0u;
         }
     }
     __syncthreads();
 
-    const int grp = threadIdx.x / S, g = g0 + grp;
+    const int grp = S == 32 ? __shfl_sync(0xffffffffu, (int)threadIdx.x / S, 0) : (int)threadIdx.x / S;
+    const int g = g0 + grp;
     Tally tally{};
-    if (grp < P && g < M.G && !Sg.done[g / M.m]) {
+    bool live = grp < P && g < M.G;
+    if (live) live = !Sg.done[g / M.m];
+    if (S == 32) live = __any_sync(0xffffffffu, live);
+    if (live) {
         unsigned char *base = smem + (size_t)grp * lay.stride;
         Stage st;
-        st.q = reinterpret_cast<longlong2 *>(base + lay.off_q);
-        st.e = reinterpret_cast<int *>(base + lay.off_e);
+        st.pk = reinterpret_cast<uint32_t *>(base + lay.off_pk);
+        st.tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
         st.bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
-        st.nbw = nbw;
-        st.mmask = M.N > kMarkBits ? (uint32_t)(kMarkBits - 1) : 0xffffffffu;
+        st.mmask = (uint32_t)(lay.marks - 1);
         const int w = g / M.m;
         const uint32_t c = Sg.slot_cfg[g];
         int E = Sg.cfg_E[c];
@@ -808,10 +898,10 @@ __device__ void sweep_block(const Model &M, const State &Sg, int g0, int P, cons
             if (tally.slow) atomicAdd(&Sg.ctl->slow, tally.slow);
             flush_ties(Sg, g, tally.tie);
             if (tally.seq) atomicAdd(&Sg.ctl->seq, (unsigned long long)tally.seq);
-#ifdef REWL_DEBUG_CHECKS
-            if (tally.bad) atomicOr(&Sg.ctl->error, ERR_BOUNDS);
-#endif
         }
+#ifdef REWL_DEBUG_CHECKS
+        if (tally.bad) atomicOr(&Sg.ctl->error, ERR_BOUNDS);
+#endif
     }
     __syncthreads();
 
@@ -819,9 +909,8 @@ __device__ void sweep_block(const Model &M, const State &Sg, int g0, int P, cons
         for (int p = 0; p < P; ++p) {
             const int gg = g0 + p;
             if (gg >= M.G || Sg.done[gg / M.m]) continue;
-            const uint32_t *lat = reinterpret_cast<const uint32_t *>(smem + (size_t)p * lay.stride + lay.off_lat);
-            uint32_t *dst_lat = Sg.spins + (size_t)Sg.slot_cfg[gg] * M.wpc;
-            for (int i = threadIdx.x; i < M.wpc; i += blockDim.x) dst_lat[i] = lat[i];
+            unstage_lattice<BITS>(M, Sg.spins + (size_t)Sg.slot_cfg[gg] * M.wpc,
+                                  reinterpret_cast<const uint32_t *>(smem + (size_t)p * lay.stride + lay.off_lat));
         }
     }
 }
@@ -841,7 +930,7 @@ __global__ void __launch_bounds__(256) batch_sweep_kernel(const InstDev *inst, c
     for (;;) {
         if (threadIdx.x == 0) next = (int)atomicAdd(queue, 1u);
         __syncthreads();
-        const int i = next;
+        const int i = __shfl_sync(0xffffffffu, next, 0);
         if (i >= n_items) break;
         const SweepItem it = items[i];
         const Model M = inst[it.inst].M;
@@ -887,12 +976,25 @@ __global__ void __launch_bounds__(256) batch_walker_kernel(const InstDev *inst, 
 #endif
 }
 
-Layout make_layout(const Model &M, int S, bool lat_global) {
+// Bits per spin of a lattice staged in shared memory: bytes, one load per spin
+// (4-bit fields take a shift and a mask more for each of a proposal's five
+// spins), unless the walker's state is so large that the wider lattice would
+// cost walkers per SM.
+constexpr int kByteStageMax = 96 * 1024;
+
+Layout make_layout(const Model &M, int S, bool lat_global, int bits);
+
+int stage_bits(const Model &M, int S, bool lat_global) {
+    if (M.bits == 8 || lat_global || S == 1) return M.bits;
+    return make_layout(M, S, false, 8).stride <= kByteStageMax ? 8 : 4;
+}
+
+Layout make_layout(const Model &M, int S, bool lat_global, int bits) {
     auto al = [](int x) { return (x + 15) & ~15; };
     Layout l{};
     int off = 0;
     if (S == 1 && lat_global) {  // every part of the walker's state in global memory
-        l.off_lgf = l.off_lat = l.off_q = l.off_e = l.off_bm = -1;
+        l.off_lgf = l.off_lat = l.off_pk = l.off_tab = l.off_bm = -1;
         l.stride = 0;
         return l;
     }
@@ -901,23 +1003,29 @@ Layout make_layout(const Model &M, int S, bool lat_global) {
     l.off_lat = -1;
     if (!lat_global) {
         l.off_lat = off;
-        off += al(M.wpc * 4);
+        off += al((M.N * bits + 31) / 32 * 4);
     }
-    if (S > 1) {  // entries past the batch: the step tree reads up to six ahead
-        l.off_q = off;
-        off += al((S + kStagePad) * 16);
-        l.off_e = off;
-        off += al((S + kStagePad) * 4);
+    l.marks = mark_entries(M.N);
+    if (off > kByteStageMax) l.marks = min(l.marks, 256);
+    // (at least the bytes per walker that decide which windows fit, so that the
+    // set of accepted configurations does not depend on the scratch below)
+    const int fits = off + (S > 1 ? al((S + 8) * 16) + al((S + 8) * 4) + al(2 * ((min(M.N, 8192) + 31) / 32) * 4) : 0);
+    if (S > 1) {
+        l.off_pk = off;
+        off += al(S * 4);
+        l.off_tab = off;
+        off += al(8 * S * 4);
         l.off_bm = off;
-        off += al(2 * ((min(M.N, kMarkBits) + 31) / 32) * 4);
+        off += al(l.marks * 4);
     }
+    off = off > fits ? off : fits;
     l.stride = al(off);
     return l;
 }
 
 template <int BITS, int S, bool LG>
 cudaError_t launch_lg(const Model &M, const State &St, const SweepPlan &p, cudaStream_t s, bool prepare) {
-    const Layout lay = make_layout(M, S, LG);
+    const Layout lay = make_layout(M, S, LG, BITS);
     if (prepare)
         return cudaFuncSetAttribute(sweep_fast_kernel<BITS, S, LG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)p.smem);
@@ -945,11 +1053,15 @@ cudaError_t dispatch_s(const Model &M, const State &St, const SweepPlan &p, cuda
 
 }  // namespace fast
 
+int sweep_bits(const Model &M, int lanes, bool lat_global) { return fast::stage_bits(M, lanes, lat_global); }
+
 size_t fast_smem_per_walker(const Model &M, int lanes, bool lat_global) {
-    return (size_t)fast::make_layout(M, lanes, lat_global).stride;
+    return (size_t)fast_layout(M, lanes, lat_global).stride;
 }
 
-Layout fast_layout(const Model &M, int lanes, bool lat_global) { return fast::make_layout(M, lanes, lat_global); }
+Layout fast_layout(const Model &M, int lanes, bool lat_global) {
+    return fast::make_layout(M, lanes, lat_global, fast::stage_bits(M, lanes, lat_global));
+}
 
 namespace {
 template <int BITS, int S>
@@ -1029,7 +1141,8 @@ int batch_walkers_ctas_per_sm(int bits, int threads) {
 }
 
 cudaError_t launch_sweep_fast(const Model &M, const State &S, const SweepPlan &p, cudaStream_t s, bool prepare) {
-    return M.bits == 8 ? fast::dispatch_s<8>(M, S, p, s, prepare) : fast::dispatch_s<4>(M, S, p, s, prepare);
+    return sweep_bits(M, p.lanes, p.lat_global != 0) == 8 ? fast::dispatch_s<8>(M, S, p, s, prepare)
+                                                          : fast::dispatch_s<4>(M, S, p, s, prepare);
 }
 
 }  // namespace rewl
