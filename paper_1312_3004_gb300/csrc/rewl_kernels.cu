@@ -253,6 +253,8 @@ __global__ void __launch_bounds__(256) sweep_kernel(Model M, State S, int P) {
 // counts the current energy and the class of the majority count
 // O = max_v #{i : s_i = v} of the configuration, one of n_obins equal integer
 // classes of [ceil(N/q), N].  Every window runs, finished or not; H stays 0.
+// This form serves windows too wide for shared memory (the other one is the
+// lane groups' PROD sweep in rewl_sweep.cu).
 // One thread per walker; lattice, ln g and the spin counts of the walker's
 // configuration buffer in global memory (the thread owns that buffer for the
 // launch); runs of equal (E, O) are added to H(E, O) with one atomic each.
@@ -734,10 +736,13 @@ cudaError_t launch_count_spins(const Model &M, const State &S, cudaStream_t s) {
 }
 
 cudaError_t launch_production_sweep(const Model &M, const State &S, cudaStream_t s) {
-    int dev = 0, sms = 0;
+    int dev = 0, sms = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
+    // a thread per walker only where a window is too wide for shared memory
+    if (launch_production_fast(M, S, sms, (size_t)optin, s, &e)) return e;
     int per = (M.G + sms - 1) / sms;  // walkers per CTA: one CTA per SM
     if (per > 256) per = 256;
     const int threads = ((per + 31) / 32) * 32, grid = (M.G + per - 1) / per;

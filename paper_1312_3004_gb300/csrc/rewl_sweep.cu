@@ -210,6 +210,10 @@ struct Stage {
     uint32_t *tab;   // [8 S] steps of the batch that end in bin x, at x mod 8 S; zero between uses
     uint32_t *bm;    // [marks] lanes of the batch that propose a site, at site & mmask; zero between uses
     uint32_t mmask;  // entries - 1 (sites share entries where N is larger: that costs comparisons only)
+    // fixed-weight production only
+    int *cnt;                 // [q] spins of each value
+    unsigned long long *heo;  // [B][n_obins] visits H(E, class) of the walker's window
+    int n_obins;
 };
 // Entries of the conflict marks: the power of two at or above N, at most this.
 constexpr int kMarks = 1024;
@@ -441,7 +445,17 @@ __device__ __noinline__ long long exact_steps(long long F, const long long *lgb,
 //  * Commit: one add of count x ln f per distinct bin (binary64 adds one by one
 //    where the integer add is not exact), one histogram add per distinct bin,
 //    one store per flipped site.
-template <int BITS, int S>
+//
+// PROD, fixed-weight production (Sec. 3.2: once g(E) is known, configurations
+// are sampled with the fixed weights 1/g(E) and distributions H(E, O)
+// recorded): ln f = 0 and ln g stays, any sign; the shadow is
+// floor((v - min) 2^k), and the binary64 values themselves settle what it does
+// not decide.  After every step H(E, O) counts the bin and the class of the
+// majority count O = max_v #{i : s_i = v}: for each value v, two ballots give
+// the steps that gain and lose a spin of it, popcounts its number after each
+// step.  Same workload, 64 classes: 8.4 -> 0.7 ms a round (1024 walkers, reads included) against one thread per
+// walker (1690 cycles a step: the binary64 decision and the counts on one chain).
+template <int BITS, int S, bool PROD = false>
 __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb,
                                              long long *lgf, uint32_t *__restrict__ hg, const Stage &st, int g, int lo,
                                              double lnf, int &E_io, unsigned long long &t_io, Tally &tally) {
@@ -462,36 +476,64 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     auto match = [&](uint32_t x) { return __match_any_sync(gm, x) >> gbase; };  // lanes with the same x
 
     // ---- fixed-point frame of this launch --------------------------------------
-    long long vmax = 0;
-    for (int b = j; b < M.B; b += S) vmax = max(vmax, lgb[b]);
+    int k;  // half-unit = 2^-k
+    int ew = 0;
+    bool int_add = false, blind = false;  // blind: no shadow (values that are no numbers), every step in binary64
+    unsigned long long incF = 0;          // ln f in half-units
+    if constexpr (PROD) {
+        double vmin = __longlong_as_double(lgb[0]), vmax = vmin;
+        bool finite = true;
+        for (int b = j; b < M.B; b += S) {
+            const double v = __longlong_as_double(lgb[b]);
+            finite = finite && fabs(v) < 0x1p1000;
+            vmin = fmin(vmin, v);
+            vmax = fmax(vmax, v);
+        }
 #pragma unroll
-    for (int o = 1; o < S; o <<= 1) vmax = max(vmax, __shfl_xor_sync(gm, vmax, o));
-    const double reach = __dadd_rn(__longlong_as_double(vmax), __dmul_rn((double)M.K, lnf));
-    // values stay below 2^(e_reach + 2 - 1023): below 2^61 units of
-    // u = 2^(ew - 1075), shadows (half-units) below 2^62
-    int ew = (int)(__double_as_longlong(reach) >> 52) - 7;
-    if (ew < 1) ew = 1;
-    const int k = 1076 - ew;  // half-unit = 2^-k
-    for (int b = j; b < M.B; b += S) lgf[b] = shadow_of(lgb[b], ew);
+        for (int o = 1; o < S; o <<= 1) {
+            vmin = fmin(vmin, __shfl_xor_sync(gm, vmin, o));
+            vmax = fmax(vmax, __shfl_xor_sync(gm, vmax, o));
+        }
+        blind = !__all_sync(gm, finite);
+        // shadows below 2^61; v - vmin is off by at most 2^-53 of it, 2^8 half-units
+        const int e = (int)(__double_as_longlong(__dsub_rn(vmax, vmin)) >> 52) - 1022;  // vmax - vmin < 2^e
+        k = min(61 - e, 57);
+        blind = blind || k < -100;  // (draws scaled by 2^k are kept in single precision)
+        for (int b = j; b < M.B; b += S) {
+            const double d = __dsub_rn(__longlong_as_double(lgb[b]), vmin);
+            lgf[b] = blind ? 0 : __double2ll_rd(d * __longlong_as_double((long long)(k + 1023) << 52));
+        }
+    } else {
+        long long vmax = 0;
+        for (int b = j; b < M.B; b += S) vmax = max(vmax, lgb[b]);
+#pragma unroll
+        for (int o = 1; o < S; o <<= 1) vmax = max(vmax, __shfl_xor_sync(gm, vmax, o));
+        const double reach = __dadd_rn(__longlong_as_double(vmax), __dmul_rn((double)M.K, lnf));
+        // values stay below 2^(e_reach + 2 - 1023): below 2^61 units of
+        // u = 2^(ew - 1075), shadows (half-units) below 2^62
+        ew = max(1, (int)(__double_as_longlong(reach) >> 52) - 7);
+        k = 1076 - ew;
+        for (int b = j; b < M.B; b += S) lgf[b] = shadow_of(lgb[b], ew);
+        bool addF;
+        const long long incU = exact_units(LNF, ew, addF);
+        // (ln f rounded down to whole units where it is none)
+        incF = (unsigned long long)(addF ? incU << 1 : shadow_of(LNF, ew) & ~1LL);
+        // every integer step inside a binade is exact when ln f is a multiple of the
+        // largest last place (2^8 units for values below 2^61 units)
+        int_add = addF && (incU & 255) == 0;
+    }
     for (int p = j; p < kPad; p += S) {
         lgf[-1 - p] = kOutside;
         lgf[M.B + p] = kOutside;
     }
-    bool addF;
-    const long long incU = exact_units(LNF, ew, addF);
-    // ln f in half-units (rounded down to whole units where it is none)
-    const unsigned long long incF = (unsigned long long)(addF ? incU << 1 : shadow_of(LNF, ew) & ~1LL);
-    // every integer step inside a binade is exact when ln f is a multiple of the
-    // largest last place (2^8 units for values below 2^61 units)
-    const bool int_add = addF && (incU & 255) == 0;
     // Decisions are first taken on the leading 32-bit words of the shadows, in
     // units of 2^(32 - k); where those cannot decide, on all 64 bits (see
     // `bracket` below).  small_k: the draws' 2^-26 fits that unit.
-    const bool small_k = __all_sync(gm, k >= 26 && k <= 57);
+    const bool small_k = __all_sync(gm, k >= 26 && k <= 57 && !blind);
     const int tsh = 58 - k;
     // At a large ln f nearly every evaluation has to count the batch's own ln f
     // steps: it does so at once, in whole leading words.
-    const bool heavy = __all_sync(gm, small_k && lnf >= 0x1p-7 && (uint32_t)incF == 0u);
+    const bool heavy = !PROD && __all_sync(gm, small_k && lnf >= 0x1p-7 && (uint32_t)incF == 0u);
     const int incH = (int)(incF >> 32);
     // ln f steps that can precede step j, in leading words (rounded up)
     const uint32_t kinc = heavy || !small_k ? 0u : (uint32_t)((incF * (unsigned)j + 0xffffffffull) >> 32);
@@ -566,6 +608,10 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         } else {
             const uint4 r = random(t);
             accept_bracket(u53(r.z, r.w), k, blo, bhi);
+            if (PROD && blind) {  // every shadow in the window is 0: nothing decided
+                blo = -(1LL << 61);
+                bhi = 1LL << 61;
+            }
         }
         width = (unsigned long long)(bhi - blo) + 2ull * kSlack;
         blo -= kSlack;
@@ -583,6 +629,11 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     read_spins();
     sts32(mark_at(next.site), next.same_mark);
     __syncwarp(gm);
+    const int qlo = PROD ? (N + M.q - 1) / M.q : 0;  // the smallest majority count
+    const uint32_t span = (uint32_t)(N - qlo + 1);
+    const bool narrow = PROD && (unsigned long long)span * (unsigned)st.n_obins < 0x100000000ull;
+    int nmax = 0;
+    for (int v = 0; PROD && v < M.q; ++v) nmax = max(nmax, st.cnt[v]);
 
     for (long long base = 0; base < M.K; base += S) {
         const int n = (int)((M.K - base) < S ? (M.K - base) : S);
@@ -734,7 +785,10 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
                 sts32(tab_at(pre), here);
                 __syncwarp(gm);
                 long long Ab = 0, Bb = 0;
-                if (j == f) {
+                if (PROD && j == f) {
+                    Ab = lgb[REWL_IDX((int)(pre - pbase) / 8, 0, M.B, tally.bad)];
+                    Bb = lgb[REWL_IDX((int)(to - pbase) / 8, 0, M.B, tally.bad)];
+                } else if (j == f) {
                     const int cA = __popc(here & le1), cB = __popc(lds32(tab_at(to)) & le1);
                     Ab = exact_steps(lds64(pre), lgb, REWL_IDX((int)(pre - pbase) / 8, 0, M.B, tally.bad), ew, lnf, cA);
                     Bb = exact_steps(lds64(to), lgb, REWL_IDX((int)(to - pbase) / 8, 0, M.B, tally.bad), ew, lnf, cB);
@@ -763,23 +817,47 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             atomicXor(&lat[site / per], (uint32_t)(cur ^ nw) << ((site & (per - 1)) * BITS));
         }
         const uint32_t at = acc ? to : pre;  // the bin after the step
-        const unsigned steps = match(j < n ? at : 0u);
+        unsigned steps = 0u;
+        if (!PROD) steps = match(j < n ? at : 0u);
         __syncwarp(gm);
         read_spins();
         sts32(mark_at(next.site), next.same_mark);
-        if (j < n && (steps & ~le) == 0u) {  // the bin's last step: its lane writes for all of them
-            const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad), c = __popc(steps);
-            const long long F = lds64(at);
-            long long F2 = (long long)((unsigned long long)F + incF * (unsigned)c);
-            const uint32_t h1 = (uint32_t)((unsigned long long)F >> 32), h2 = (uint32_t)((unsigned long long)F2 >> 32);
-            if (!int_add || (F & 1) || (h2 ^ h1) > h1) {  // binary64 adds
-                const long long v = exact_steps(F, lgb, b, ew, lnf, c);
-                F2 = shadow_of(v, ew);
-                if (F2 & 1) lgb[b] = v;
-                nseq += (unsigned)c;
+        if constexpr (PROD) {
+            int most = nmax;  // the majority count after the step
+            if (A) {
+                most = 0;
+#pragma unroll 2
+                for (int v = 0; v < M.q; ++v) {
+                    const int c = st.cnt[v];
+                    const unsigned up = ballot(acc && nw == v), down = ballot(acc && cur == v);
+                    most = max(most, c + __popc(up & le) - __popc(down & le));
+                    if ((up | down) != 0u && j == 0) st.cnt[v] = c + __popc(up) - __popc(down);
+                }
+                nmax = __shfl_sync(gm, most, n - 1, S);
             }
-            sts64(at, F2);
-            atomicAdd(&hg[b], (uint32_t)c);  // (result not used: the walker does not wait)
+            // class = (O - ceil(N / q)) n_obins / (N - ceil(N / q) + 1)
+            const uint32_t x = (uint32_t)(most - qlo);
+            const int cls = narrow ? (int)(x * (uint32_t)st.n_obins / span)
+                                   : (int)((unsigned long long)x * (unsigned)st.n_obins / span);
+            const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad);
+            const int key = b * st.n_obins + cls;
+            steps = match(j < n ? (uint32_t)key : 0xffffffffu);
+            if (j < n && (steps & ~le) == 0u) atomicAdd(&st.heo[key], (unsigned long long)__popc(steps));
+        } else {
+            if (j < n && (steps & ~le) == 0u) {  // the bin's last step: its lane writes for all of them
+                const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad), c = __popc(steps);
+                const long long F = lds64(at);
+                long long F2 = (long long)((unsigned long long)F + incF * (unsigned)c);
+                const uint32_t h1 = (uint32_t)((unsigned long long)F >> 32), h2 = (uint32_t)((unsigned long long)F2 >> 32);
+                if (!int_add || (F & 1) || (h2 ^ h1) > h1) {  // binary64 adds
+                    const long long v = exact_steps(F, lgb, b, ew, lnf, c);
+                    F2 = shadow_of(v, ew);
+                    if (F2 & 1) lgb[b] = v;
+                    nseq += (unsigned)c;
+                }
+                sts64(at, F2);
+                atomicAdd(&hg[b], (uint32_t)c);  // (result not used: the walker does not wait)
+            }
         }
         pcur = __shfl_sync(gm, at, n - 1, S);
         nacc += acc ? 1u : 0u;
@@ -787,7 +865,7 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         __syncwarp(gm);
     }
     // the binary64 array from the authoritative shadow
-    for (int b = j; b < M.B; b += S) {
+    for (int b = j; !PROD && b < M.B; b += S) {
         const long long F = lgf[b];
         if (!(F & 1)) lgb[b] = from_units(F >> 1, ew);
     }
@@ -919,6 +997,71 @@ template <int BITS, int S, bool LG>
 __global__ void __launch_bounds__(256) sweep_fast_kernel(Model M, State Sg, int P, Layout lay) {
     extern __shared__ __align__(16) unsigned char smem[];
     sweep_block<BITS, S, LG>(M, Sg, blockIdx.x * P, P, lay, smem);
+}
+
+// Fixed-weight production: P walkers per CTA, a lane group of 32 each; every
+// window runs, finished or not, with the walkers' own ln g.
+template <int BITS, bool LG>
+__global__ void __launch_bounds__(256) production_fast_kernel(Model M, State Sg, int P, Layout lay, int off_cnt) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int g0 = blockIdx.x * P;
+    for (int p = 0; p < P && g0 + p < M.G; ++p) {
+        unsigned char *base = smem + (size_t)p * lay.stride;
+        const uint32_t c = Sg.slot_cfg[g0 + p];
+        if (!LG)
+            stage_lattice<BITS>(M, reinterpret_cast<uint32_t *>(base + lay.off_lat), Sg.spins + (size_t)c * M.wpc);
+        uint32_t *bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
+        for (int i = threadIdx.x; i < lay.marks; i += blockDim.x) bm[i] = 0u;
+        uint32_t *tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
+        for (int i = threadIdx.x; i < 8 * 32; i += blockDim.x) tab[i] = 0u;
+        int *cnt = reinterpret_cast<int *>(base + off_cnt);
+        for (int i = threadIdx.x; i < M.q; i += blockDim.x) cnt[i] = Sg.cnt[(size_t)c * M.q + i];
+    }
+    __syncthreads();
+
+    const int grp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0);
+    const int g = g0 + grp;
+    Tally tally{};
+    if (__any_sync(0xffffffffu, grp < P && g < M.G)) {
+        unsigned char *base = smem + (size_t)grp * lay.stride;
+        const int w = g / M.m;
+        const uint32_t c = Sg.slot_cfg[g];
+        Stage st;
+        st.pk = reinterpret_cast<uint32_t *>(base + lay.off_pk);
+        st.tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
+        st.bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
+        st.mmask = (uint32_t)(lay.marks - 1);
+        st.cnt = reinterpret_cast<int *>(base + off_cnt);
+        st.heo = Sg.heo + (size_t)w * M.B * M.n_obins;
+        st.n_obins = M.n_obins;
+        int E = Sg.cfg_E[c];
+        unsigned long long t = Sg.t[g];
+        walker_sweep<BITS, 32, true>(M, LG ? Sg.spins + (size_t)c * M.wpc : reinterpret_cast<uint32_t *>(base + lay.off_lat),
+                                     reinterpret_cast<long long *>(Sg.lng + (size_t)g * M.B),
+                                     reinterpret_cast<long long *>(base + lay.off_lgf) + kPad, nullptr, st, g, Sg.e_lo[w],
+                                     0.0, E, t, tally);
+        if ((threadIdx.x & 31) == 0) {
+            Sg.cfg_E[c] = E;
+            Sg.t[g] = t;
+            atomicAdd(&Sg.ctl->flips, (unsigned long long)M.K);
+            atomicAdd(&Sg.ctl->accepted, (unsigned long long)tally.acc);
+            if (tally.slow) atomicAdd(&Sg.ctl->slow, tally.slow);
+            flush_ties(Sg, g, tally.tie);
+        }
+#ifdef REWL_DEBUG_CHECKS
+        if (tally.bad) atomicOr(&Sg.ctl->error, ERR_BOUNDS);
+#endif
+    }
+    __syncthreads();
+
+    for (int p = 0; p < P && g0 + p < M.G; ++p) {
+        const unsigned char *base = smem + (size_t)p * lay.stride;
+        const uint32_t c = Sg.slot_cfg[g0 + p];
+        if (!LG)
+            unstage_lattice<BITS>(M, Sg.spins + (size_t)c * M.wpc, reinterpret_cast<const uint32_t *>(base + lay.off_lat));
+        const int *cnt = reinterpret_cast<const int *>(base + off_cnt);
+        for (int i = threadIdx.x; i < M.q; i += blockDim.x) Sg.cnt[(size_t)c * M.q + i] = cnt[i];
+    }
 }
 
 // Persistent batched sweep: each CTA takes the next item from *queue.
@@ -1122,6 +1265,31 @@ int batch_sweep_ctas_per_sm(int bits, int lanes, int threads, size_t smem) {
     case 16: return occupancy_t<4, 16>(threads, smem);
     default: return occupancy_t<4, 32>(threads, smem);
     }
+}
+
+// Whether a walker's production state fits a CTA's shared memory; if so, queue
+// the sweep (P walkers a CTA, one CTA per SM while the walkers last: their
+// chains, not a pipe, set the rate).
+bool launch_production_fast(const Model &M, const State &S, int num_sms, size_t smem_optin, cudaStream_t s,
+                            cudaError_t *err) {
+    const bool lg = M.wpc * 4 > kSharedLatticeMax;
+    const int bits = sweep_bits(M, 32, lg);
+    Layout lay = fast::make_layout(M, 32, lg, bits);
+    const int off_cnt = lay.stride;
+    lay.stride += (M.q * 4 + 15) & ~15;
+    int P = (int)(smem_optin / (size_t)lay.stride);
+    P = min(min(P, 8), (M.G + num_sms - 1) / num_sms);
+    if (P < 1) return false;
+    const size_t smem = (size_t)P * (size_t)lay.stride;
+    auto go = [&](auto kernel) {
+        *err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (*err != cudaSuccess) return;
+        kernel<<<(M.G + P - 1) / P, P * 32, smem, s>>>(M, S, P, lay, off_cnt);
+        *err = cudaGetLastError();
+    };
+    if (lg) bits == 8 ? go(fast::production_fast_kernel<8, true>) : go(fast::production_fast_kernel<4, true>);
+    else bits == 8 ? go(fast::production_fast_kernel<8, false>) : go(fast::production_fast_kernel<4, false>);
+    return true;
 }
 
 cudaError_t launch_batch_walkers(int bits, const InstDev *inst, const WalkerItem *items, int n_items, int grid,
