@@ -120,8 +120,8 @@ enum : int { SWEEP_REFERENCE = 0, SWEEP_FAST = 1 };
 struct Layout {
     int stride;                 // bytes per walker (multiple of 16)
     int off_lgf, off_lat;       // byte offsets: ln g shadow (with sentinels), lattice
-    int off_pk, off_tab, off_bm;  // proposals, steps by bin and conflict marks of a batch (lane groups)
-    int marks;                  // entries of the conflict marks (a power of two)
+    int off_ring, off_pk, off_tab, off_bm;  // proposals drawn ahead, proposals, lanes by bin and conflict marks of a batch (lane groups)
+    int marks;                  // entries of the conflict marks (a power of two where below N)
 };
 
 // One instance of a batch, as the batched kernels see it.

@@ -24,6 +24,7 @@
 //    iteration over the whole batch (walker_sweep below).
 //  * S = 1: a thread per walker, one step after another (walker_sweep_1).
 #include <cstdint>
+#include <type_traits>
 
 #include "rewl_internal.cuh"
 
@@ -47,6 +48,23 @@ __device__ __forceinline__ uint4 philox_rounds(uint32_t c0, uint32_t c1, uint32_
 // 20 three-input logic operations a block).
 __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const uint32_t (&rk)[20]) {
     return philox_rounds(c0, c1, c2, c3, [&](int w, int r) { return rk[2 * r + w]; });
+}
+// C blocks of one key, counter words t[c] (low, high) and c2, interleaved so that
+// the rounds of one hide the latency of another.
+template <int C>
+__device__ __forceinline__ void philox_blocks(const unsigned long long (&t)[C], uint32_t c2, uint32_t c3,
+                                              const uint32_t (&rk)[20], uint4 (&x)[C]) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) x[c] = make_uint4((uint32_t)t[c], (uint32_t)(t[c] >> 32), c2, c3);
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const unsigned long long a = 0xD2511F53ull * x[c].x, b = 0xCD9E8D57ull * x[c].z;
+            x[c] = make_uint4((uint32_t)(b >> 32) ^ x[c].y ^ rk[2 * r], (uint32_t)b,
+                              (uint32_t)(a >> 32) ^ x[c].w ^ rk[2 * r + 1], (uint32_t)a);
+        }
+    }
 }
 // A thread per walker: the keys of different walkers differ, and 20 registers
 // for them would cost warps per SM.
@@ -206,22 +224,25 @@ __device__ __forceinline__ unsigned group_mask() {
 
 // Per-walker scratch of the lane group in shared memory (S > 1 only).
 struct Stage {
-    uint32_t *pk;    // [S] proposal k as conflicting lanes read it: site | new value << 20
-    uint32_t *tab;   // [8 S] steps of the batch that end in bin x, at x mod 8 S; zero between uses
-    uint32_t *bm;    // [marks] lanes of the batch that propose a site, at site & mmask; zero between uses
-    uint32_t mmask;  // entries - 1 (sites share entries where N is larger: that costs comparisons only)
+    uint2 *ring;     // [kAhead S] proposals drawn ahead: site | new value index << 20; -ln u
+    uint32_t *pk;    // [2 S] proposal k as touched lanes read it: site | new value << 20; lanes at its mark
+    uint32_t *tab;   // [8 S] lanes that start from bin x, at x mod 8 S; zero between uses
+    uint8_t *bm;     // [marks] a lane of the batch that proposes a site, at the site's entry (kNoLane: none)
+    uint32_t mmask;  // all bits, or entries - 1 where sites share entries (that costs comparisons only)
     // fixed-weight production only
     int *cnt;                 // [q] spins of each value
     unsigned long long *heo;  // [B][n_obins] visits H(E, class) of the walker's window
     int n_obins;
 };
-// Entries of the conflict marks: the power of two at or above N, at most this.
-constexpr int kMarks = 1024;
-inline int mark_entries(int N) {
-    int e = 32;
-    while (e < N && e < kMarks) e <<= 1;
-    return e;
-}
+// Entries of the conflict marks: one per site up to kMarks sites.
+constexpr int kMarks = 8192;
+constexpr uint32_t kNoLane = 255u;
+// ln f from which a lane group counts the batch's own ln f steps in every
+// evaluation (about 60 cycles each) instead of leaving the steps they could
+// decide, about 500 ln f a batch of 32, to the full comparison (about 1000 cycles).
+constexpr double kCountLnf = 0x1p-12;
+constexpr int kCrowded = 300;
+constexpr int kAhead = 4;  // batches drawn at a time
 // Half-units by which D in a batch can miss the true difference beyond the
 // floors of shadow_of: up to 32 adds on either bin, each rounded by at most
 // half a last place (2^8 half-units for values below 2^61 units) and, for an
@@ -400,6 +421,39 @@ __device__ __noinline__ long long exact_steps(long long F, const long long *lgb,
     return __double_as_longlong(a);
 }
 
+// The shadow after c ln f steps from F where integers give the reference's
+// binary64 sums although the plain add does not apply; false where they do not.
+// F2: on entry F + c ln f in whole units.
+//  - ln f a multiple of the largest last place (int_add): only a step into the
+//    next binade can round, and only if the sum has bits below that binade's last
+//    place; the steps leave those bits as they are, so the last sum shows them.
+//  - another ln f (the 1/t rule's bins / steps): inside a binade every step adds
+//    the same whole number of last places, ln f rounded to them, unless ln f lies
+//    half-way between two (then the sum's parity decides).
+__device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, int ew, bool int_add, long long &F2) {
+    if (F & 1) return false;
+    if (int_add) {
+        const int sh = 11 - __clzll(F2 >> 1);
+        return sh <= 0 || ((F2 >> 1) & ((1LL << sh) - 1)) == 0;
+    }
+    const int sh = 11 - __clzll(F >> 1);  // the last place of F's binade is 2^sh units
+    if (F == 0 || sh < 0 || LNF < (1LL << 52)) return false;
+    const int s = sh + ew - (int)(LNF >> 52);  // and 2^s last places of ln f
+    const long long mf = (LNF & kMant) | kHidden;
+    long long inc = 0;
+    if (s >= 0 && s <= 54) {
+        const long long rest = mf & ((1LL << s) - 1), half = s > 0 ? 1LL << (s - 1) : 1;
+        if (rest == half) return false;
+        inc = (mf >> s) + (rest > half ? 1 : 0);
+    } else if (s < 0) {
+        if (s < -8) return false;
+        inc = mf << -s;
+    }
+    if (inc >= 1LL << 52) return false;
+    F2 = F + ((inc << sh) * c << 1);
+    return __clzll(F2) == __clzll(F);
+}
+
 // S > 1 lanes per walker: batches of S steps, lane j owning step j.
 //
 // A step's outcome depends on the earlier steps of its batch only through the
@@ -415,15 +469,19 @@ __device__ __noinline__ long long exact_steps(long long F, const long long *lgb,
 // confirming evaluation included.
 //
 // What bounds it: the latency of one dependent chain per walker (with 7 walkers
-// per SM nothing else is near its limit), so every part is chosen for its
-// latency.  Measured on GB300, in cycles with their use: popcount 24 (four of
-// them 56), ballot 17, match 38, shared load 34, store-then-load 42,
-// atomic-then-load 99, leading-zero count 27, a branch on a vote about 45.
-// Hence matches and plain stores instead of shared atomics, and one branch per
-// evaluation.  q = 10, L = 80, 1024 walkers, 10^4 steps each: 1.17 -> 0.72 ms a
-// round in the first rounds (ln f = 1) and 1.10 -> 0.55 ms at ln f = 2^-20,
-// against the step trees that were here before (the decisions of the next five
-// steps at a time, 275 cycles a step).
+// per SM a batch takes 1740 cycles against 1600 with one walker on the SM alone,
+// and the pipes are a third busy), so every part is chosen for its latency.
+// Measured on GB300, in cycles with their use: popcount 24 (four of them 56),
+// ballot 17 (four 33), match 41 and 11 more per distinct value, shared load 34,
+// store-then-load 42, atomic-then-load 99, leading-zero count 27, a branch on a
+// vote about 45.  Hence ballots and plain stores instead of shared atomics, one
+// branch per evaluation, and the random numbers of four batches at a time (600 ->
+// 290 cycles a batch).  Cycles per batch of 32 at ln f = 2^-20: draws 290,
+// proposals 410, 1.5 evaluations 400, commit 550; at ln f = 1: 4.9 evaluations
+// 1560.  q = 10, L = 80, 1024 walkers, 10^4 steps each, sweep alone: 1.10 -> 0.58 ms
+// in the first rounds (ln f = 1) and 1.03 -> 0.40 ms at ln f = 2^-20, against the
+// step trees that were here before (the decisions of the next five steps at a
+// time, 275 cycles a step).
 //
 //  * The bin before step j: the batch's start plus the accepted energy changes
 //    of the lanes before it; from four ballots (the bit planes of the changes,
@@ -431,12 +489,10 @@ __device__ __noinline__ long long exact_steps(long long F, const long long *lgb,
 //  * ln f steps added inside the batch: at a large ln f every evaluation counts
 //    them, otherwise only when one of the at most j that precede step j could
 //    decide.  The steps before j that ended in a bin are the lanes 1 .. j that
-//    start from it: for the old bin a match of the lanes' bins, for the new one
-//    that match read through a table by bin (mod 8 S: the path spans at most
-//    4 S + 4 bins either way).
-//  * Flips: every lane leaves the lanes that propose its site at the site's
-//    entry of a table and reads the entries of its four neighbours; the energy
-//    change of a lane that others touch is recomputed from the spins at the
+//    start from it: from the bit planes of the lanes' bins, by ballots.
+//  * Flips: a byte per site names a lane that proposes it, and every lane reads
+//    its own site's and those of its four neighbours; the energy change of a
+//    lane that others touch is recomputed from the spins at the
 //    start of the batch and the flips of the accepted touching lanes, in order,
 //    whenever those change.
 //  * A draw inside its bracket is settled when everything before it is final:
@@ -473,7 +529,6 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     const uint32_t qm1 = (uint32_t)(M.q - 1);
     const long long LNF = __double_as_longlong(lnf);
     auto ballot = [&](bool p) { return __ballot_sync(gm, p) >> gbase; };
-    auto match = [&](uint32_t x) { return __match_any_sync(gm, x) >> gbase; };  // lanes with the same x
 
     // ---- fixed-point frame of this launch --------------------------------------
     int k;  // half-unit = 2^-k
@@ -530,11 +585,11 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     // units of 2^(32 - k); where those cannot decide, on all 64 bits (see
     // `bracket` below).  small_k: the draws' 2^-26 fits that unit.
     const bool small_k = __all_sync(gm, k >= 26 && k <= 57 && !blind);
-    const int tsh = 58 - k;
-    // At a large ln f nearly every evaluation has to count the batch's own ln f
-    // steps: it does so at once, in whole leading words.
-    const bool heavy = !PROD && __all_sync(gm, small_k && lnf >= 0x1p-7 && (uint32_t)incF == 0u);
-    const int incH = (int)(incF >> 32);
+    const int tsh = small_k ? 58 - k : 0;
+    // At a large ln f many evaluations have to count the batch's own ln f steps:
+    // they all do, in leading words (loose: with up to 32 units for what those cut off).
+    const bool heavy = !PROD && __all_sync(gm, small_k && lnf >= kCountLnf);
+    const int incH = (int)(incF >> 32), loose = heavy && (uint32_t)incF != 0u ? 32 : 0;
     // ln f steps that can precede step j, in leading words (rounded up)
     const uint32_t kinc = heavy || !small_k ? 0u : (uint32_t)((incF * (unsigned)j + 0xffffffffull) >> 32);
     __syncwarp(gm);
@@ -546,19 +601,34 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     uint32_t pcur = pbase + (uint32_t)(E_io - lo) * 8u;  // shared address of the current bin's shadow
     unsigned int nacc = 0, nseq = 0;
     auto lds32 = [](uint32_t a) { return *reinterpret_cast<const uint32_t *>(__cvta_shared_to_generic(a)); };
-    auto sts32 = [](uint32_t a, uint32_t v) { *reinterpret_cast<uint32_t *>(__cvta_shared_to_generic(a)) = v; };
     auto lead = [&](uint32_t a) { return (int)lds32(a + 4u); };  // leading word of a shadow
+    auto sts32 = [](uint32_t a, uint32_t v) { *reinterpret_cast<uint32_t *>(__cvta_shared_to_generic(a)) = v; };
     // the entry of tab that stands for the bin whose shadow is at shared address a
     auto tab_at = [&](uint32_t a) { return tbase + ((a >> 1) & (uint32_t)(32 * S - 4)); };
-    // conflict marks: the lanes of the batch that propose a site, at the site's
-    // entry (sites share entries where N is larger than the table)
-    const uint32_t mbytes = st.mmask << 2;
-    auto mark_at = [&](int s) { return mbase + (((uint32_t)s << 2) & mbytes); };
-    const bool shared_marks = (uint32_t)N > st.mmask + 1u;
+    // Lanes whose x has the low seven bits of this lane's y, from bit planes by
+    // ballots.  Bins a path of one batch visits, or proposes from its second step
+    // on, are less than 128 apart.
+    auto planes = [&](uint32_t x, unsigned (&p)[7]) {
+#pragma unroll
+        for (int b = 0; b < 7; ++b) p[b] = ballot((x >> b) & 1u);
+    };
+    auto equal = [&](const unsigned (&p)[7], uint32_t y) {
+        unsigned eq = ~0u;
+#pragma unroll
+        for (int b = 0; b < 7; ++b) eq &= (y >> b) & 1u ? p[b] : ~p[b];
+        return eq;
+    };
+    auto mark_at = [&](int s) { return mbase + ((uint32_t)s & st.mmask); };
+    const bool shared_marks = st.mmask != 0xffffffffu;
+    // On small lattices most batches propose some site twice: the lanes of each
+    // site are matched ahead, with the draws (300 cycles for about 25 sites, under
+    // the waits of a batch); elsewhere they are compared one by one when it occurs.
+    const bool crowded = N <= kCrowded;
+    auto lds8 = [](uint32_t a) { return (uint32_t)*reinterpret_cast<const uint8_t *>(__cvta_shared_to_generic(a)); };
+    auto sts8 = [](uint32_t a, uint32_t v) { *reinterpret_cast<uint8_t *>(__cvta_shared_to_generic(a)) = (uint8_t)v; };
 
     // The part of a proposal that needs no state: site, neighbours, new value,
-    // T = -ln u in 2^-26 (kTiny: u < 2^-24, only D < 0 is decided by it), the
-    // lanes that propose the same site or share its entry of the marks, and
+    // T = -ln u in 2^-26 (kTiny: u < 2^-24, only D < 0 is decided by it), and
     // [blo, blo + bw): the leading-word differences that do not decide.  The
     // true difference D 2^-32 lies strictly within 1 of the difference of the
     // leading words, kSlack is far below a leading word's unit, and out of the
@@ -567,31 +637,44 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     struct Draw {
         int site, v, T, blo;
         uint32_t bw;
-        unsigned same_site, same_mark;
+        unsigned twins;  // lanes that propose the same site (found ahead on small lattices)
         Site4 nb;
     };
     auto random = [&](unsigned long long t) {
         return philox((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)g, DOM_WL, M.rk);
     };
-    auto draw = [&](unsigned long long t) {
-        const uint4 r = random(t);
+    // The random part of the next kAhead batches (from step t on), into the ring.
+    auto draw_ahead = [&](unsigned long long t0) {
+        unsigned long long t[kAhead];
+        uint4 r[kAhead];
+#pragma unroll
+        for (int c = 0; c < kAhead; ++c) t[c] = t0 + (unsigned long long)(c * S + j);
+        philox_blocks<kAhead>(t, (uint32_t)g, DOM_WL, M.rk, r);
+#pragma unroll
+        for (int c = 0; c < kAhead; ++c) {
+            // as accept_bracket, in integers: u from its leading 27 bits and the rest
+            // (relative error below 2^-23), -ln u from lg2.approx (absolute or relative
+            // error at most 2^-22, times ln 2) and rounded to 2^-26: together below
+            // (Lf + 1) 2^-21; the margin is (Lf + 1) 2^-18
+            const float uf = fmaf((float)(r[c].z & ~31u), 0x1p-32f, (float)r[c].w * 0x1p-59f);
+            float l2;
+            asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l2) : "f"(uf));
+            const int T = r[c].z < 256u ? kTiny : __float2int_rn(l2 * -0x1.62e43p+25f);  // below 2^31 for u >= 2^-24
+            st.ring[c * S + j] = make_uint2(__umulhi(r[c].x, (uint32_t)N) | __umulhi(r[c].y, qm1) << 20, (uint32_t)T);
+        }
+    };
+    auto drawn = [&](int c) {  // this lane's proposal of batch c of the ring
+        const uint2 w = st.ring[c * S + j];
         Draw d;
-        d.site = (int)__umulhi(r.x, (uint32_t)N);
-        d.v = (int)__umulhi(r.y, qm1);
+        d.site = (int)(w.x & 0xfffffu);
+        d.v = (int)(w.x >> 20);
+        d.T = (int)w.y;
         d.nb = nbrs(d.site, L, N, M.divL);
-        d.same_site = match((uint32_t)d.site);
-        d.same_mark = match(mark_at(d.site));
-        // as accept_bracket, in integers: u from its leading 27 bits and the rest
-        // (relative error below 2^-23), -ln u from lg2.approx (absolute or relative
-        // error at most 2^-22, times ln 2) and rounded to 2^-26: together below
-        // (Lf + 1) 2^-21; the margin is (Lf + 1) 2^-18
-        const float uf = fmaf((float)(r.z & ~31u), 0x1p-32f, (float)r.w * 0x1p-59f);
-        float l2;
-        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l2) : "f"(uf));
-        d.T = r.z < 256u ? kTiny : __float2int_rn(l2 * -0x1.62e43p+25f);  // below 2^31 for u >= 2^-24
+        d.twins = bit;
+        if (crowded) d.twins = __match_any_sync(gm, d.site) >> gbase;
         const int mg = (d.T >> 18) + 260;  // (Lf + 1) 2^-18, rounded up
-        d.blo = ((d.T - mg) >> tsh) - 1;
-        d.bw = (uint32_t)(((d.T + mg) >> tsh) + 3 - d.blo);
+        d.blo = ((d.T - mg) >> tsh) - 1 - loose;
+        d.bw = (uint32_t)(((d.T + mg) >> tsh) + 3 + loose - d.blo);
         if (d.T == kTiny || !small_k) {
             d.blo = small_k ? -2 : -0x7fffffff;
             d.bw = 0xfffffff0u;
@@ -617,7 +700,9 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         blo -= kSlack;
     };
 
-    Draw next = draw(t_io + (unsigned long long)j);
+    draw_ahead(t_io);
+    Draw next = drawn(0);  // (a lane reads back its own entries only)
+    int ahead = 0;         // the batch of the ring that `next` holds
     int cur0, sr0, sl0, sd0, su0;
     auto read_spins = [&]() {
         cur0 = spin_get<BITS>(lat, next.site);
@@ -627,7 +712,7 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         su0 = spin_get<BITS>(lat, next.nb.u);
     };
     read_spins();
-    sts32(mark_at(next.site), next.same_mark);
+    sts8(mark_at(next.site), (uint32_t)j);
     __syncwarp(gm);
     const int qlo = PROD ? (N + M.q - 1) / M.q : 0;  // the smallest majority count
     const uint32_t span = (uint32_t)(N - qlo + 1);
@@ -635,8 +720,9 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     int nmax = 0;
     for (int v = 0; PROD && v < M.q; ++v) nmax = max(nmax, st.cnt[v]);
 
-    for (long long base = 0; base < M.K; base += S) {
-        const int n = (int)((M.K - base) < S ? (M.K - base) : S);
+    long long left = M.K;
+    for (;;) {
+        const int n = left < S ? (int)left : S;
         // ---- lane j prepares proposal t + j against the lattice as it is --------
         // (its spins were read, and its site marked, at the end of the last batch)
         Draw d = next;
@@ -646,8 +732,8 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         int dE = (int)(sr0 == cur) + (int)(sl0 == cur) + (int)(sd0 == cur) + (int)(su0 == cur) - (int)(sr0 == nw) -
                  (int)(sl0 == nw) - (int)(sd0 == nw) - (int)(su0 == nw);
         // earlier lanes whose flip would change this proposal
-        unsigned touch = (d.same_mark | lds32(mark_at(nb.r)) | lds32(mark_at(nb.l)) | lds32(mark_at(nb.d)) |
-                          lds32(mark_at(nb.u))) & lt;
+        unsigned touch = 0u, twins = d.twins;  // ... ; lanes that propose the same site
+        const uint32_t m0 = lds8(mark_at(site)), mr = lds8(mark_at(nb.r)), ml = lds8(mark_at(nb.l)), md = lds8(mark_at(nb.d)), mu = lds8(mark_at(nb.u));
         if (n < S && j >= n) {  // past the launch's last step: never accepted
             d.blo = (int)0x80000000;
             d.bw = 0u;
@@ -660,24 +746,46 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         // bit planes of the energy changes (two's complement)
         unsigned q0 = ballot(dE & 1), q1 = ballot(dE & 2), q2 = ballot(dE & 4), q3 = ballot(dE & 8);
         unsigned A = ballot(D0 < d.blo);  // the steps that accept, as presently known
-        unsigned fl = ballot(touch != 0u);
+        // (without two lanes at one entry every mark names the only lane there)
+        unsigned fl = ballot(m0 != (uint32_t)j || min(min(mr, ml), min(md, mu)) < (uint32_t)j);
         // the state-free part of the next batch's proposals: independent
         // instructions for the waits of this batch
-        next = draw(t_io + (unsigned long long)(S + j));
+        if (++ahead == kAhead) {
+            draw_ahead(t_io + S);
+            ahead = 0;
+        }
+        next = drawn(ahead);
         __syncwarp(gm);
-        sts32(mark_at(site), 0u);
+        sts8(mark_at(site), kNoLane);
         if (fl) {
+            unsigned there = twins;  // lanes at this site's entry
+            for (unsigned rest = crowded ? 0u : ballot(m0 != (uint32_t)j); rest;) {
+                const int f = __ffs((int)rest) - 1;
+                const int sf = __shfl_sync(gm, site, f, S);
+                const unsigned t = ballot(site == sf);
+                const unsigned e = shared_marks ? ballot(mark_at(site) == mark_at(sf)) : t;
+                if (t & bit) twins = t;
+                if (e & bit) there = e;
+                rest &= ~t;
+            }
             st.pk[j] = (uint32_t)site | ((uint32_t)nw << 20);
+            st.pk[S + j] = there;
+            __syncwarp(gm);
+            touch = there;
+            if (mr != kNoLane) touch |= st.pk[S + mr];
+            if (ml != kNoLane) touch |= st.pk[S + ml];
+            if (md != kNoLane) touch |= st.pk[S + md];
+            if (mu != kNoLane) touch |= st.pk[S + mu];
+            touch &= lt;
             if (shared_marks) {  // keep the lanes that do touch
-                __syncwarp(gm);
                 unsigned real = 0u;
                 for (unsigned rest = touch; rest; rest &= rest - 1u) {
                     const int ps = (int)(st.pk[__ffs((int)rest) - 1] & 0xfffffu);
                     if (ps == site || ps == nb.r || ps == nb.l || ps == nb.d || ps == nb.u) real |= rest & (0u - rest);
                 }
                 touch = real;
-                fl = ballot(touch != 0u);
             }
+            fl = ballot(touch != 0u);
         }
 
         // ---- evaluations until nothing changes -----------------------------------
@@ -726,10 +834,18 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             pre = (uint32_t)max(pmin, min((int)p, pmax));
             to = pre + (uint32_t)(dE * 8);
         };
-        // ln f steps the path adds to step j's new bin before it, less those it
-        // adds to its old one: the lanes that start from a bin, through tab
-        auto counted = [&]() {
-            const unsigned here = match(pre);
+        // ln f steps the path adds to step j's new bin before it, and to its old
+        // one: the lanes 1 .. j that start from them
+        auto counted = [&](int &cA, int &cB) {
+            unsigned p[7];
+            planes((pre - pcur) >> 3, p);
+            cA = __popc(equal(p, (pre - pcur) >> 3) & le1);
+            cB = __popc(equal(p, (to - pcur) >> 3) & le1);
+        };
+        // the same for every evaluation at a large ln f: in a fifth of the
+        // instructions, by a match (11 cycles per distinct bin) and a table
+        auto counted_now = [&]() {
+            const unsigned here = __match_any_sync(gm, pre) >> gbase;
             const uint32_t slot = tab_at(pre);
             __syncwarp(gm);
             sts32(slot, here);
@@ -739,13 +855,14 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             sts32(slot, 0u);
             return __popc(there & le1) - __popc(here & le1);
         };
-        int D;
+        unsigned open;  // steps that the leading words do not decide
         if (heavy) {
             for (;;) {
                 if (fl) reflip();
                 place();
-                D = lead(to) - lead(pre) + incH * counted();
+                const int D = lead(to) - lead(pre) + incH * counted_now();
                 const unsigned A2 = ballot(D < d.blo);
+                open = ballot((uint32_t)(D - d.blo) < d.bw);
                 if (A2 == A && moved == 0u) break;
                 A = A2;
             }
@@ -753,15 +870,15 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             for (;;) {
                 if (fl) reflip();
                 place();
-                D = lead(to) - lead(pre);
+                const int D = lead(to) - lead(pre);
                 const unsigned A2 = ballot(D < d.blo);
+                open = ballot((uint32_t)(D - blo2) < bw2);
                 if (A2 == A && moved == 0u) break;
                 A = A2;
             }
         }
-        if (ballot(heavy ? (uint32_t)(D - d.blo) < d.bw : (uint32_t)(D - blo2) < bw2)) {
-            // a step the leading words do not decide: on from here with all 64 bits
-            // and the batch's own ln f steps
+        if (open) {
+            // on from here with all 64 bits and the batch's own ln f steps
             long long b64;
             unsigned long long w64;
             bracket(d.T, t_io + (unsigned long long)j, b64, w64);
@@ -769,8 +886,10 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             for (;;) {
                 if (fl) reflip();
                 place();
+                int cA, cB;
+                counted(cA, cB);
                 const unsigned long long D64 = (unsigned long long)lds64(to) - (unsigned long long)lds64(pre) +
-                                               incF * (unsigned long long)(long long)counted();
+                                               incF * (unsigned long long)(long long)(cB - cA);
                 const unsigned A2 = (ballot(j < n && (long long)D64 < b64) & ~fm) | fv;
                 const unsigned um = ballot(j < n && D64 - (unsigned long long)b64 < w64) & ~fm;
                 if (A2 != A || moved != 0u) {
@@ -780,21 +899,13 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
                 if (um == 0u) break;
                 // the first undecided step: the reference's test in binary64
                 const int f = __ffs((int)um) - 1;
-                const unsigned here = match(pre);
-                __syncwarp(gm);
-                sts32(tab_at(pre), here);
-                __syncwarp(gm);
                 long long Ab = 0, Bb = 0;
-                if (PROD && j == f) {
-                    Ab = lgb[REWL_IDX((int)(pre - pbase) / 8, 0, M.B, tally.bad)];
-                    Bb = lgb[REWL_IDX((int)(to - pbase) / 8, 0, M.B, tally.bad)];
-                } else if (j == f) {
-                    const int cA = __popc(here & le1), cB = __popc(lds32(tab_at(to)) & le1);
-                    Ab = exact_steps(lds64(pre), lgb, REWL_IDX((int)(pre - pbase) / 8, 0, M.B, tally.bad), ew, lnf, cA);
-                    Bb = exact_steps(lds64(to), lgb, REWL_IDX((int)(to - pbase) / 8, 0, M.B, tally.bad), ew, lnf, cB);
+                if (j == f) {
+                    const int ia = REWL_IDX((int)(pre - pbase) / 8, 0, M.B, tally.bad);
+                    const int ib = REWL_IDX((int)(to - pbase) / 8, 0, M.B, tally.bad);
+                    Ab = PROD ? lgb[ia] : exact_steps(lds64(pre), lgb, ia, ew, lnf, cA);
+                    Bb = PROD ? lgb[ib] : exact_steps(lds64(to), lgb, ib, ew, lnf, cB);
                 }
-                __syncwarp(gm);
-                sts32(tab_at(pre), 0u);
                 Ab = __shfl_sync(gm, Ab, f, S);
                 Bb = __shfl_sync(gm, Bb, f, S);
                 const unsigned long long tf = t_io + (unsigned long long)f;
@@ -812,16 +923,16 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         // reads run under the ln g updates
         const bool acc = (A & bit) != 0u;
         if (BITS == 8) {  // the site's last accepted value stays
-            if (acc && (d.same_site & A & ~le) == 0u) reinterpret_cast<uint8_t *>(lat)[site] = (uint8_t)nw;
+            if (acc && (twins & A & ~le) == 0u) reinterpret_cast<uint8_t *>(lat)[site] = (uint8_t)nw;
         } else if (acc) {
             atomicXor(&lat[site / per], (uint32_t)(cur ^ nw) << ((site & (per - 1)) * BITS));
         }
         const uint32_t at = acc ? to : pre;  // the bin after the step
-        unsigned steps = 0u;
-        if (!PROD) steps = match(j < n ? at : 0u);
+        unsigned steps = 0u;  // those that ended in this lane's bin
+        if (!PROD) steps = __match_any_sync(gm, j < n ? at : 0u) >> gbase;
         __syncwarp(gm);
         read_spins();
-        sts32(mark_at(next.site), next.same_mark);
+        sts8(mark_at(next.site), (uint32_t)j);
         if constexpr (PROD) {
             int most = nmax;  // the majority count after the step
             if (A) {
@@ -841,19 +952,25 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
                                    : (int)((unsigned long long)x * (unsigned)st.n_obins / span);
             const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad);
             const int key = b * st.n_obins + cls;
-            steps = match(j < n ? (uint32_t)key : 0xffffffffu);
-            if (j < n && (steps & ~le) == 0u) atomicAdd(&st.heo[key], (unsigned long long)__popc(steps));
+            // one add per run of equal keys, by its last step
+            const int after = __shfl_down_sync(gm, key, 1, S);
+            const bool ends = j < n && (j == n - 1 || after != key);
+            const unsigned before = ballot(ends) & lt;
+            if (ends) atomicAdd(&st.heo[key], (unsigned long long)(before ? j - 31 + __clz((int)before) : j + 1));
         } else {
+            const long long F = lds64(at);
+            const int c = __popc(steps);
             if (j < n && (steps & ~le) == 0u) {  // the bin's last step: its lane writes for all of them
-                const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad), c = __popc(steps);
-                const long long F = lds64(at);
+                const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad);
                 long long F2 = (long long)((unsigned long long)F + incF * (unsigned)c);
                 const uint32_t h1 = (uint32_t)((unsigned long long)F >> 32), h2 = (uint32_t)((unsigned long long)F2 >> 32);
-                if (!int_add || (F & 1) || (h2 ^ h1) > h1) {  // binary64 adds
-                    const long long v = exact_steps(F, lgb, b, ew, lnf, c);
-                    F2 = shadow_of(v, ew);
-                    if (F2 & 1) lgb[b] = v;
-                    nseq += (unsigned)c;
+                if (!int_add || (F & 1) || (h2 ^ h1) > h1) {
+                    if (!whole_steps(F, c, LNF, ew, int_add, F2)) {  // binary64 adds
+                        const long long v = exact_steps(F, lgb, b, ew, lnf, c);
+                        F2 = shadow_of(v, ew);
+                        if (F2 & 1) lgb[b] = v;
+                        nseq += (unsigned)c;
+                    }
                 }
                 sts64(at, F2);
                 atomicAdd(&hg[b], (uint32_t)c);  // (result not used: the walker does not wait)
@@ -862,7 +979,9 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         pcur = __shfl_sync(gm, at, n - 1, S);
         nacc += acc ? 1u : 0u;
         t_io += (unsigned long long)n;
+        left -= n;
         __syncwarp(gm);
+        if (left <= 0) break;
     }
     // the binary64 array from the authoritative shadow
     for (int b = j; !PROD && b < M.B; b += S) {
@@ -938,7 +1057,7 @@ __device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int
                                 Sg.spins + (size_t)Sg.slot_cfg[g] * M.wpc);
         if (S > 1) {
             uint32_t *bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
-            for (int i = threadIdx.x; i < lay.marks; i += blockDim.x) bm[i] = 0u;
+            for (int i = threadIdx.x; i < lay.marks / 4; i += blockDim.x) bm[i] = 0xffffffffu;
             uint32_t *tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
             for (int i = threadIdx.x; i < 8 * S; i += blockDim.x) tab[i] = 0u;
         }
@@ -954,10 +1073,11 @@ __device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int
     if (live) {
         unsigned char *base = smem + (size_t)grp * lay.stride;
         Stage st;
+        st.ring = reinterpret_cast<uint2 *>(base + lay.off_ring);
         st.pk = reinterpret_cast<uint32_t *>(base + lay.off_pk);
         st.tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
-        st.bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
-        st.mmask = (uint32_t)(lay.marks - 1);
+        st.bm = base + lay.off_bm;
+        st.mmask = lay.marks >= M.N ? 0xffffffffu : (uint32_t)(lay.marks - 1);
         const int w = g / M.m;
         const uint32_t c = Sg.slot_cfg[g];
         int E = Sg.cfg_E[c];
@@ -994,7 +1114,7 @@ __device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int
 }
 
 template <int BITS, int S, bool LG>
-__global__ void __launch_bounds__(256) sweep_fast_kernel(Model M, State Sg, int P, Layout lay) {
+__global__ void __launch_bounds__(256, 1) sweep_fast_kernel(Model M, State Sg, int P, Layout lay) {
     extern __shared__ __align__(16) unsigned char smem[];
     sweep_block<BITS, S, LG>(M, Sg, blockIdx.x * P, P, lay, smem);
 }
@@ -1011,9 +1131,7 @@ __global__ void __launch_bounds__(256) production_fast_kernel(Model M, State Sg,
         if (!LG)
             stage_lattice<BITS>(M, reinterpret_cast<uint32_t *>(base + lay.off_lat), Sg.spins + (size_t)c * M.wpc);
         uint32_t *bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
-        for (int i = threadIdx.x; i < lay.marks; i += blockDim.x) bm[i] = 0u;
-        uint32_t *tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
-        for (int i = threadIdx.x; i < 8 * 32; i += blockDim.x) tab[i] = 0u;
+        for (int i = threadIdx.x; i < lay.marks / 4; i += blockDim.x) bm[i] = 0xffffffffu;
         int *cnt = reinterpret_cast<int *>(base + off_cnt);
         for (int i = threadIdx.x; i < M.q; i += blockDim.x) cnt[i] = Sg.cnt[(size_t)c * M.q + i];
     }
@@ -1027,10 +1145,11 @@ __global__ void __launch_bounds__(256) production_fast_kernel(Model M, State Sg,
         const int w = g / M.m;
         const uint32_t c = Sg.slot_cfg[g];
         Stage st;
+        st.ring = reinterpret_cast<uint2 *>(base + lay.off_ring);
         st.pk = reinterpret_cast<uint32_t *>(base + lay.off_pk);
         st.tab = reinterpret_cast<uint32_t *>(base + lay.off_tab);
-        st.bm = reinterpret_cast<uint32_t *>(base + lay.off_bm);
-        st.mmask = (uint32_t)(lay.marks - 1);
+        st.bm = base + lay.off_bm;
+        st.mmask = lay.marks >= M.N ? 0xffffffffu : (uint32_t)(lay.marks - 1);
         st.cnt = reinterpret_cast<int *>(base + off_cnt);
         st.heo = Sg.heo + (size_t)w * M.B * M.n_obins;
         st.n_obins = M.n_obins;
@@ -1137,7 +1256,7 @@ Layout make_layout(const Model &M, int S, bool lat_global, int bits) {
     Layout l{};
     int off = 0;
     if (S == 1 && lat_global) {  // every part of the walker's state in global memory
-        l.off_lgf = l.off_lat = l.off_pk = l.off_tab = l.off_bm = -1;
+        l.off_lgf = l.off_lat = l.off_ring = l.off_pk = l.off_tab = l.off_bm = -1;
         l.stride = 0;
         return l;
     }
@@ -1148,18 +1267,20 @@ Layout make_layout(const Model &M, int S, bool lat_global, int bits) {
         l.off_lat = off;
         off += al((M.N * bits + 31) / 32 * 4);
     }
-    l.marks = mark_entries(M.N);
-    if (off > kByteStageMax) l.marks = min(l.marks, 256);
+    l.marks = M.N <= kMarks ? al(M.N) : kMarks;
+    if (off > kByteStageMax) l.marks = 512;
     // (at least the bytes per walker that decide which windows fit, so that the
     // set of accepted configurations does not depend on the scratch below)
     const int fits = off + (S > 1 ? al((S + 8) * 16) + al((S + 8) * 4) + al(2 * ((min(M.N, 8192) + 31) / 32) * 4) : 0);
     if (S > 1) {
+        l.off_ring = off;
+        off += al(kAhead * S * 8);
         l.off_pk = off;
-        off += al(S * 4);
+        off += al(2 * S * 4);
         l.off_tab = off;
         off += al(8 * S * 4);
         l.off_bm = off;
-        off += al(l.marks * 4);
+        off += l.marks;
     }
     off = off > fits ? off : fits;
     l.stride = al(off);

@@ -37,14 +37,14 @@ def test_last_batch_of_a_launch(K, lanes):
     same((10, 8, 3, 0.75, 3, 1e-6, 0.8, K, 5), 4, 6, lanes)
 
 
-@pytest.mark.parametrize("L", [3, 4, 31, 32, 33, 47])  # sites per entry of the conflict marks: 1 up to 32 x 32
+@pytest.mark.parametrize("L", [3, 4, 17, 18, 32, 47, 90, 91])  # twin sites found ahead up to 300 sites; own conflict marks up to 8192
 @pytest.mark.parametrize("q,bits", [(2, 8), (10, 4), (20, 8)])
 def test_lattice_sizes(L, q, bits):
     h = 1 if L < 5 else 3
     same((q, L, h, 0.75, 2, 1e-6, 0.8, 3000, 7), bits, 3, 32)
 
 
-@pytest.mark.parametrize("lnf", [0.0, 1.0, 2.0**-6, 2.0**-7, 2.0**-8, 2.0**-20, 2.0**-45, 1e-3, 0.3, 3.7])
+@pytest.mark.parametrize("lnf", [0.0, 1.0, 2.0**-7, 2.0**-12, 2.0**-13, 2.0**-20, 2.0**-45, 1e-3, 1e-5, 0.3, 3.7])
 @pytest.mark.parametrize("L", [6, 20])
 def test_ln_f(lnf, L):
     """counted at once, counted where it matters, not at all; whole units of the
@@ -55,11 +55,12 @@ def test_ln_f(lnf, L):
     same((5, L, 2, 0.75, 3, 1e-300, 0.999, 2000, 11), 4, 4, 32, prepare)
 
 
-@pytest.mark.parametrize("scale,offset", [(1.0, 0.0), (0.125, 0.0), (1e-9, 0.0), (1.0, 1e6), (1.0, 3e9), (1.0, 1e11), (1.0, 1e15)])
+@pytest.mark.parametrize("scale,offset", [(1.0, 0.0), (0.125, 0.0), (1e-9, 0.0), (1.0, 1e6), (1.0, 3e9), (1.0, 1e11), (1.0, 1e13), (1.0, 1e15)])
 @pytest.mark.parametrize("lnf", [0.0, 2.0**-10, 1.0])
 def test_range_of_ln_g(scale, offset, lnf):
     """shadows whose unit is finer and coarser than the draws' (leading words
-    that cannot decide send every decision to 64 bits)"""
+    that cannot decide send every decision to 64 bits); ln f half-way between two
+    last places"""
     def prepare(r):
         b = np.arange(r.B)
         r.set("lng", scale * (40.0 * np.sin(b / 17.0) ** 2 + 0.37 * b) + offset)
