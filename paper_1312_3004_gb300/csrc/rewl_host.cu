@@ -772,6 +772,7 @@ rewl_status rewl_get_field(rewl_t h, int field, void *out, size_t bytes) {
     rewl_status st = field_geometry(h, field, &dev, &need);
     if (st) return st;
     if (bytes != need) return fail(REWL_ERR_ARG, "field %d needs %zu bytes, got %zu", field, need, bytes);
+    rewl::host::touch_pages(out, bytes);
     if (field == REWL_FIELD_SPINS) {
         uint8_t *tmp = nullptr;
         REWL_CUDA(cudaMallocAsync((void **)&tmp, need, h->stream));
@@ -780,13 +781,15 @@ rewl_status rewl_get_field(rewl_t h, int field, void *out, size_t bytes) {
         cudaFreeAsync(tmp, h->stream);
         if (e != cudaSuccess) return fail(REWL_ERR_CUDA, "spins: %s", cudaGetErrorString(e));
     } else if (field == REWL_FIELD_ENERGY) {
-        std::vector<uint32_t> slot((size_t)h->M.G);
-        std::vector<int32_t> cfgE((size_t)h->M.G);
-        REWL_CUDA(cudaMemcpyAsync(slot.data(), h->S.slot_cfg, slot.size() * 4, cudaMemcpyDeviceToHost, h->stream));
-        REWL_CUDA(cudaMemcpyAsync(cfgE.data(), h->S.cfg_E, cfgE.size() * 4, cudaMemcpyDeviceToHost, h->stream));
+        // cfg_E and slot_cfg lie side by side in the state: one copy for both
+        const size_t from = h->parts[1].off, off = h->parts[2].off - from;
+        std::vector<unsigned char> both(off + h->parts[2].bytes);
+        REWL_CUDA(cudaMemcpyAsync(both.data(), (const char *)h->dmem + from, both.size(), cudaMemcpyDeviceToHost, h->stream));
         REWL_CUDA(cudaStreamSynchronize(h->stream));
+        const int32_t *cfgE = (const int32_t *)both.data();
+        const uint32_t *slot = (const uint32_t *)(both.data() + off);
         int32_t *o = (int32_t *)out;
-        for (size_t g = 0; g < slot.size(); ++g) o[g] = cfgE[slot[g]];
+        for (size_t g = 0; g < (size_t)h->M.G; ++g) o[g] = cfgE[slot[g]];
         return REWL_OK;
     } else {
         REWL_CUDA(cudaMemcpyAsync(out, dev, need, cudaMemcpyDeviceToHost, h->stream));
@@ -837,6 +840,7 @@ rewl_status rewl_save(rewl_t h, void *buf, size_t *len) {
         return REWL_OK;
     }
     if (*len < need) return fail(REWL_ERR_ARG, "buffer of %zu bytes < %zu", *len, need);
+    rewl::host::touch_pages(buf, need);
     unsigned char *dst = (unsigned char *)buf + sizeof(SaveHeader);
     for (size_t i = 0; i < h->parts.size(); ++i) {
         const auto &p = h->parts[i];

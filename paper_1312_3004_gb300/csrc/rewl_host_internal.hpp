@@ -37,6 +37,24 @@ cudaError_t dev_alloc(DevBlock &b, size_t bytes);
 void dev_free(DevBlock &b);
 void set_allocator(void *(*alloc)(size_t, void *), void (*free_fn)(void *, void *), void *ctx);
 
+// Write to every page of a caller's result buffer that a copy from the device is
+// about to fill.  Fresh pageable memory that the device reaches through the
+// host's page tables is otherwise faulted in by the copy, one page at a time
+// (16 MB of fresh 64 KB pages: 10 - 13 ms; touched first: under 2 ms).
+// Only pageable host memory: any other pointer is left to the copy, which takes
+// or refuses it.
+inline void touch_pages(void *p, size_t bytes) {
+    if (bytes < (size_t)(256 << 10)) return;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (a.type != cudaMemoryTypeUnregistered) return;
+    volatile unsigned char *c = (volatile unsigned char *)p;
+    for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
+}
+
 // A named range on the host timeline of a profiler (NVTX; free when none is attached).
 struct Range {
     explicit Range(const char *name) { nvtxRangePushA(name); }

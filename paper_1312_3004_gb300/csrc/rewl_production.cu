@@ -81,6 +81,7 @@ rewl_status rewl_production_histogram(rewl_t h, unsigned long long *out, size_t 
     if (!h->M.production) return rewl::host::fail(REWL_ERR_STATE, "no production started (rewl_production_start)");
     const size_t need = (size_t)h->M.h * h->M.B * (size_t)h->M.n_obins;
     if (len != need) return rewl::host::fail(REWL_ERR_ARG, "len %zu != h * (W + 1) * n_obins = %zu", len, need);
+    rewl::host::touch_pages(out, need * 8);
     PROD_CUDA(cudaMemcpyAsync(out, h->S.heo, need * 8, cudaMemcpyDeviceToHost, h->stream));
     PROD_CUDA(cudaStreamSynchronize(h->stream));
     return REWL_OK;
