@@ -345,7 +345,7 @@ rewl_status rewl_batch_create_ext(const rewl_params *jobs, int n, int spin_bits,
  * what it computes).  Times the batch's candidate configurations -- spin
  * packing 4 or 8 bits (when spin_bits was 0 and every q <= 16), walkers as lane
  * groups of 32 with 36, 72 or 110 KB of shared memory per sweep CTA (when
- * lanes was 0 and the walkers fit) or as a thread each with 128 or 256
+ * lanes was 0 and the walkers fit) or as a thread each with 32 or 128
  * threads per CTA -- each over `rounds` rounds (after one round that settles
  * it), by CUDA events on the batch's stream and the WL proposals counted, and
  * leaves the batch in the fastest one.  The rounds it runs are ordinary rounds

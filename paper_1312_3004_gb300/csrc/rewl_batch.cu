@@ -37,7 +37,7 @@ struct Config {
     int bits = 8;           // spins per configuration word: 4 or 8 bits each
     int lanes = 32;         // 32: lane groups, state staged in shared memory; 1: a thread per walker
     int cta_kb = 72;        // lanes 32: shared memory per sweep CTA (walkers per CTA follow)
-    int threads = 256;      // lanes 1: threads per CTA
+    int threads = 32;       // lanes 1: threads per CTA (a warp: 1775 of them spread evenly over 152 SMs)
 };
 
 struct SweepClass {
@@ -424,7 +424,7 @@ rewl_status rewl_batch_autotune(rewl_batch_t b, int rounds, rewl_tune_entry *ent
                     cands.push_back(c);
                 }
             } else {
-                for (int t : {128, 256}) {
+                for (int t : {32, 128}) {
                     c.threads = t;
                     cands.push_back(c);
                 }

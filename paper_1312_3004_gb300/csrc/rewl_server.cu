@@ -34,7 +34,7 @@ namespace {
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-constexpr int kWalkerThreads = 128;  // threads per CTA of the thread-per-walker sweep
+constexpr int kWalkerThreads = 32;   // threads per CTA of the thread-per-walker sweep
 constexpr long long kTuneMinWalkers = 512;  // below this, lane groups (a walker's chain sets the rate)
 
 // First-fit allocator over one device arena (offsets in bytes, 256-aligned).

@@ -66,14 +66,6 @@ __device__ __forceinline__ void philox_blocks(const unsigned long long (&t)[C], 
         }
     }
 }
-// A thread per walker: the keys of different walkers differ, and 20 registers
-// for them would cost warps per SM.
-__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1) {
-    return philox_rounds(c0, c1, c2, c3, [&](int w, int r) {
-        return w == 0 ? k0 + (uint32_t)r * 0x9E3779B9u : k1 + (uint32_t)r * 0xBB67AE85u;
-    });
-}
-
 template <int BITS>
 __device__ __forceinline__ int spin_get(const uint32_t *w, int s) {
     if (BITS == 8) return reinterpret_cast<const uint8_t *>(w)[s];
@@ -211,10 +203,6 @@ __device__ __forceinline__ void flush_ties(const State &S, int g, const TieRec &
     if (tie.n > 2ull) atomicAdd(&S.ctl->ties, tie.n - 2ull);
 }
 
-__device__ __noinline__ long long exact_add(long long A, double lnf) {
-    return __double_as_longlong(__dadd_rn(__longlong_as_double(A), lnf));
-}
-
 template <int S>
 __device__ __forceinline__ unsigned group_mask() {
     if (S >= 32) return 0xffffffffu;
@@ -267,20 +255,6 @@ __device__ __forceinline__ long long from_units(long long F, int ew) {
     return ((long long)(ew + sh) << 52) | (m & kMant);
 }
 
-// Round an exact shadow (tag 0) to 53 significant bits, ties to even: the
-// binary64 rounding of a ln f step that entered the next binade.
-__device__ __forceinline__ long long round_shadow(long long F2) {
-    long long F = F2 >> 1;
-    const int sh = 11 - __clzll(F);
-    if (sh <= 0) return F2;
-    const long long ulp = 1LL << sh, r = F & (ulp - 1);
-    if (r == 0) return F2;
-    const long long half = ulp >> 1;
-    F -= r;
-    if (r > half || (r == half && ((F >> sh) & 1))) F += ulp;
-    return F << 1;
-}
-
 // 64-bit access to the shadow array by 32-bit shared address.  Lanes of a
 // group see each other's writes only across a __syncwarp.
 __device__ __forceinline__ long long lds64(uint32_t a) {
@@ -290,126 +264,35 @@ __device__ __forceinline__ void sts64(uint32_t a, long long v) {
     *reinterpret_cast<long long *>(__cvta_shared_to_generic(a)) = v;
 }
 
-// One lane per walker: the steps one after another, each proposal drawn (and
-// its spins read) while the previous step waits for its ln g shadow; a
-// proposal whose site or neighbours the previous step flipped is re-read.
-// The frame, the shadow, the bracket and the exact fallbacks are those of
-// walker_sweep below.
-template <int BITS>
-__device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb, long long *lgf,
-                               uint32_t *__restrict__ hg, int g, int lo, double lnf, int &E_io,
-                               unsigned long long &t_io, Tally &tally) {
-    const int N = M.N, L = M.L;
-    constexpr int per = 32 / BITS;
-    const uint32_t qm1 = (uint32_t)(M.q - 1);
-    const long long LNF = __double_as_longlong(lnf);
-    long long vmax = 0;
-    for (int b = 0; b < M.B; ++b) vmax = max(vmax, lgb[b]);
-    const double reach = __dadd_rn(__longlong_as_double(vmax), __dmul_rn((double)M.K, lnf));
-    int ew = (int)(__double_as_longlong(reach) >> 52) - 7;
-    if (ew < 1) ew = 1;
-    const int k = 1076 - ew;
-    for (int b = 0; b < M.B; ++b) lgf[b] = shadow_of(lgb[b], ew);
-    for (int p = 0; p < kPad; ++p) {
-        lgf[-1 - p] = kOutside;
-        lgf[M.B + p] = kOutside;
+// What both forms of the sweep share: the fixed-point frame of a launch and the
+// brackets of -ln u on it.
+//
+// T = -ln u in 2^-26 (kTiny: u < 2^-24, only D < 0 is decided by it): as
+// accept_bracket, in integers -- u from its leading 27 bits and the rest (relative
+// error below 2^-23), -ln u from lg2.approx (absolute or relative error at most
+// 2^-22, times ln 2) and rounded to 2^-26: together below (Lf + 1) 2^-21; the
+// margin is (Lf + 1) 2^-18.
+constexpr int kTiny = 0x7fffffff;
+__device__ __forceinline__ int minus_ln(uint32_t hi, uint32_t lo) {
+    const float uf = fmaf((float)(hi & ~31u), 0x1p-32f, (float)lo * 0x1p-59f);
+    float l2;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l2) : "f"(uf));
+    return hi < 256u ? kTiny : __float2int_rn(l2 * -0x1.62e43p+25f);  // below 2^31 for u >= 2^-24
+}
+// Decisions are first taken on the leading 32-bit words of the shadows, in units
+// of 2^(32 - k): [blo, blo + bw) are the differences of leading words that do not
+// decide (the true difference D 2^-32 lies strictly within 1 of the difference of
+// the leading words, kSlack is far below a leading word's unit, and out of the
+// window the difference is at least 2^30 - 2, above every T at tsh = 58 - k >= 1).
+// small_k: the draws' 2^-26 fits that unit, 26 <= k <= 57; loose: more units.
+__device__ __forceinline__ void lead_bracket(int T, bool small_k, int tsh, int loose, int &blo, uint32_t &bw) {
+    const int mg = (T >> 18) + 260;  // (Lf + 1) 2^-18, rounded up
+    blo = ((T - mg) >> tsh) - 1 - loose;
+    bw = (uint32_t)(((T + mg) >> tsh) + 3 + loose - blo);
+    if (T == kTiny || !small_k) {
+        blo = small_k ? -2 : -0x7fffffff;
+        bw = 0xfffffff0u;
     }
-    bool addF;
-    const long long incU = exact_units(LNF, ew, addF);
-    const long long incF = incU << 1;
-    const bool int_add = addF && (incU & 255) == 0;
-
-    struct Prop {
-        int site, v, cur, sr, sl, sd, su;
-        Site4 nb;
-        longlong2 th;
-        unsigned long long U;
-    };
-    auto draw = [&](unsigned long long tt, Prop &p) {
-        const uint4 r = philox((uint32_t)tt, (uint32_t)(tt >> 32), (uint32_t)g, DOM_WL, M.key0, M.key1);
-        p.site = (int)__umulhi(r.x, (uint32_t)N);
-        p.v = (int)__umulhi(r.y, qm1);
-        p.nb = nbrs(p.site, L, N, M.divL);
-        p.cur = spin_get<BITS>(lat, p.site);
-        p.sr = spin_get<BITS>(lat, p.nb.r);
-        p.sl = spin_get<BITS>(lat, p.nb.l);
-        p.sd = spin_get<BITS>(lat, p.nb.d);
-        p.su = spin_get<BITS>(lat, p.nb.u);
-        p.U = u53(r.z, r.w);
-        accept_bracket(p.U, k, p.th.x, p.th.y);
-    };
-    // The current bin's shadow AF and its visits since the walker came are kept
-    // in registers, and written when the walker leaves the bin.
-    int Eo = E_io - lo;
-    long long AF = lgf[REWL_IDX(Eo, 0, M.B, tally.bad)];
-    uint32_t visits = 0;
-    unsigned int nacc = 0;
-    int flipped = -1;  // site the previous step flipped
-    Prop cp;
-    draw(t_io, cp);
-    for (long long i = 0; i < M.K; ++i) {
-        if (flipped >= 0 && (flipped == cp.site || flipped == cp.nb.r || flipped == cp.nb.l || flipped == cp.nb.d ||
-                             flipped == cp.nb.u)) {
-            cp.cur = spin_get<BITS>(lat, cp.site);
-            cp.sr = spin_get<BITS>(lat, cp.nb.r);
-            cp.sl = spin_get<BITS>(lat, cp.nb.l);
-            cp.sd = spin_get<BITS>(lat, cp.nb.d);
-            cp.su = spin_get<BITS>(lat, cp.nb.u);
-        }
-        const int nw = cp.v + (cp.v >= cp.cur);
-        const int dE = (int)(cp.sr == cp.cur) + (int)(cp.sl == cp.cur) + (int)(cp.sd == cp.cur) + (int)(cp.su == cp.cur) -
-                       (int)(cp.sr == nw) - (int)(cp.sl == nw) - (int)(cp.sd == nw) - (int)(cp.su == nw);
-        const int En = Eo + dE;
-        const long long BF = dE == 0 ? AF : lgf[REWL_IDX(En, -kPad, M.B + kPad, tally.bad)];  // beyond: kOutside
-        Prop np;
-        if (i + 1 < M.K) draw(t_io + (unsigned long long)i + 1ull, np);
-        const long long D = BF - AF;
-        bool acc = D < cp.th.x;
-        if (!acc && D < cp.th.y) {  // inside the bracket (never beyond the window)
-            tally.slow += 1;
-            const long long Ab = (AF & 1) ? lgb[REWL_IDX(Eo, 0, M.B, tally.bad)] : from_units(AF >> 1, ew);
-            const long long Bb = (BF & 1) ? lgb[REWL_IDX(En, 0, M.B, tally.bad)] : from_units(BF >> 1, ew);
-            acc = dE == 0 ? true : exact_accept(Ab, Bb, cp.U, &tally.tie, t_io + (unsigned long long)i);
-        }
-        const long long cur = acc ? BF : AF;  // with dE = 0 both are the current shadow
-        const int Eb2 = acc ? En : Eo;
-        long long AF2 = cur + incF;
-        if (!int_add || (cur & 1)) {  // ln g(E) += ln f in binary64
-            tally.seq += 1;
-            const long long Ab = (cur & 1) ? lgb[REWL_IDX(Eb2, 0, M.B, tally.bad)] : from_units(cur >> 1, ew);
-            const long long A2 = exact_add(Ab, lnf);
-            lgb[REWL_IDX(Eb2, 0, M.B, tally.bad)] = A2;
-            AF2 = shadow_of(A2, ew);
-        } else {
-            const uint32_t hc = (uint32_t)((unsigned long long)cur >> 32);
-            const uint32_t h2 = (uint32_t)((unsigned long long)AF2 >> 32);
-            if ((h2 ^ hc) > hc) AF2 = round_shadow(AF2);  // into the next binade
-        }
-        // (atomics whose result is not used: the walker does not wait for them)
-        if (Eb2 != Eo) {  // leaving the bin: its value and visits go to memory
-            lgf[REWL_IDX(Eo, 0, M.B, tally.bad)] = AF;
-            atomicAdd(&hg[REWL_IDX(Eo, 0, M.B, tally.bad)], visits);
-            visits = 0;
-        }
-        ++visits;
-        Eo = Eb2;
-        AF = AF2;
-        if (acc) {
-            atomicXor(&lat[cp.site / per], (uint32_t)(cp.cur ^ nw) << ((cp.site & (per - 1)) * BITS));
-            ++nacc;
-        }
-        flipped = acc ? cp.site : -1;
-        cp = np;
-    }
-    lgf[Eo] = AF;
-    atomicAdd(&hg[Eo], visits);
-    t_io += (unsigned long long)M.K;
-    for (int b = 0; b < M.B; ++b) {
-        const long long F = lgf[b];
-        if (!(F & 1)) lgb[b] = from_units(F >> 1, ew);
-    }
-    tally.acc += nacc;
-    E_io = Eo + lo;
 }
 
 // The exact binary64 value of a bin after `count` more ln f steps of the batch:
@@ -452,6 +335,217 @@ __device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, i
     if (inc >= 1LL << 52) return false;
     F2 = F + ((inc << sh) * c << 1);
     return __clzll(F2) == __clzll(F);
+}
+
+// One lane per walker, its state in global memory: the steps one after another,
+// each proposal drawn (and its spins read) while the previous step waits for its
+// ln g shadow; a spin that the previous step flipped is replaced in registers.
+//
+// What bounds it: the instructions of a step and how few warps there are to
+// overlap their latencies (about 12 per SM on 2048 instances).  Hence leading-word
+// decisions, brackets in 32-bit integers, round keys kept in registers, plain
+// stores to the lattice (the thread owns it) and the current bin's shadow and
+// visits in registers until the walker leaves the bin.  The passes over all bins
+// before and after the steps are taken by the warp together, one walker after
+// another, so that the lanes' loads lie side by side (3.1 -> @W2@ ms on 2048
+// instances).  Every thread of a warp calls, live or not.  2048 instances, 56,784
+// walkers, 10^4 steps: 16.1 -> @W1@ ms a round.
+struct Slow1 {  // what the rare parts of a step need
+    long long *lgb;
+    double lnf;
+    int ew, k;
+    bool small_k;
+    unsigned int slow = 0, seq = 0;
+};
+// The decision with all 64 bits, then in binary64; r: the step's random words.
+__device__ __noinline__ bool decide_1(Slow1 &s, long long AF, long long BF, int a, int b, int T, uint4 r, TieRec *tie,
+                                      unsigned long long t) {
+    long long blo, bhi;
+    if (s.small_k && T != kTiny) {
+        const int mg = (T >> 18) + 260;
+        blo = (long long)(T - mg) << (s.k - 26);
+        bhi = (long long)(T + mg) << (s.k - 26);
+    } else {
+        accept_bracket(u53(r.z, r.w), s.k, blo, bhi);
+    }
+    const long long D = BF - AF;
+    if (D < blo - kSlack) return true;
+    if (D >= bhi + kSlack) return false;
+    s.slow += 1;
+    return exact_accept(exact_steps(AF, s.lgb, a, s.ew, 0.0, 0), exact_steps(BF, s.lgb, b, s.ew, 0.0, 0), u53(r.z, r.w), tie,
+                        t);
+}
+__device__ __noinline__ long long add_1(Slow1 &s, long long F, int b, long long F2, bool int_add) {
+    if (whole_steps(F, 1, __double_as_longlong(s.lnf), s.ew, int_add, F2)) return F2;
+    s.seq += 1;
+    const long long v = exact_steps(F, s.lgb, b, s.ew, s.lnf, 1);
+    s.lgb[b] = v;
+    return shadow_of(v, s.ew);
+}
+
+constexpr int kInFlight = 8;  // loads of such a pass in flight per lane
+
+template <int BITS>
+__device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb, long long *lgf,
+                               uint32_t *__restrict__ hg, int g, int lo, double lnf, int &E_io,
+                               unsigned long long &t_io, Tally &tally, bool live) {
+    const int N = M.N, L = M.L;
+    constexpr int per = 32 / BITS;
+    const uint32_t qm1 = (uint32_t)(M.q - 1), divL = M.divL;
+    const long long LNF = __double_as_longlong(lnf);
+    const int lane = (int)(threadIdx.x & 31u);
+    const unsigned lanes = __ballot_sync(0xffffffffu, live);
+    auto of = [&](auto *p, int w) {  // lane w's pointer
+        return reinterpret_cast<decltype(p)>(__shfl_sync(0xffffffffu, (unsigned long long)p, w));
+    };
+    long long vmax = 0;
+    for (unsigned rest = lanes; rest; rest &= rest - 1u) {
+        const int w = __ffs((int)rest) - 1, B = __shfl_sync(0xffffffffu, M.B, w);
+        const long long *v = of(lgb, w);
+        long long top = 0;
+        for (int b0 = lane; b0 < B; b0 += 32 * kInFlight) {
+            long long x[kInFlight];
+#pragma unroll
+            for (int i = 0; i < kInFlight; ++i) x[i] = b0 + 32 * i < B ? v[b0 + 32 * i] : 0;
+#pragma unroll
+            for (int i = 0; i < kInFlight; ++i) top = max(top, x[i]);
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+        if (lane == w) vmax = top;
+    }
+    const double reach = __dadd_rn(__longlong_as_double(vmax), __dmul_rn((double)M.K, lnf));
+    Slow1 rare;
+    rare.lgb = lgb;
+    rare.lnf = lnf;
+    rare.ew = max(1, (int)(__double_as_longlong(reach) >> 52) - 7);
+    rare.k = 1076 - rare.ew;
+    rare.small_k = rare.k >= 26 && rare.k <= 57;
+    const bool small_k = rare.small_k;
+    const int tsh = small_k ? 58 - rare.k : 0;
+    for (unsigned rest = lanes; rest; rest &= rest - 1u) {
+        const int w = __ffs((int)rest) - 1, B = __shfl_sync(0xffffffffu, M.B, w), e = __shfl_sync(0xffffffffu, rare.ew, w);
+        const long long *v = of(lgb, w);
+        long long *f = of(lgf, w);
+        for (int b0 = lane; b0 < B; b0 += 32 * kInFlight) {
+            long long x[kInFlight];
+#pragma unroll
+            for (int i = 0; i < kInFlight; ++i) x[i] = b0 + 32 * i < B ? v[b0 + 32 * i] : 0;
+#pragma unroll
+            for (int i = 0; i < kInFlight; ++i)
+                if (b0 + 32 * i < B) f[b0 + 32 * i] = shadow_of(x[i], e);
+        }
+        if (lane < kPad) {
+            f[-1 - lane] = kOutside;
+            f[B + lane] = kOutside;
+        }
+    }
+    __syncwarp();
+    bool addF;
+    const long long incU = exact_units(LNF, rare.ew, addF);
+    const unsigned long long incF = (unsigned long long)(addF ? incU << 1 : shadow_of(LNF, rare.ew) & ~1LL);
+    const bool int_add = addF && (incU & 255) == 0;
+    uint32_t rk[20];
+#pragma unroll
+    for (uint32_t r = 0; r < 10; ++r) {
+        rk[2 * r] = M.key0 + r * 0x9E3779B9u;
+        rk[2 * r + 1] = M.key1 + r * 0xBB67AE85u;
+    }
+
+    struct Prop {
+        int site, v, cur, sr, sl, sd, su, T, blo;
+        uint32_t bw;
+        Site4 nb;
+    };
+    auto random = [&](unsigned long long t) {
+        return philox((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)g, DOM_WL, rk);
+    };
+    auto draw = [&](unsigned long long t, Prop &p) {
+        const uint4 r = random(t);
+        p.site = (int)__umulhi(r.x, (uint32_t)N);
+        p.v = (int)__umulhi(r.y, qm1);
+        p.nb = nbrs(p.site, L, N, divL);
+        p.cur = spin_get<BITS>(lat, p.site);
+        p.sr = spin_get<BITS>(lat, p.nb.r);
+        p.sl = spin_get<BITS>(lat, p.nb.l);
+        p.sd = spin_get<BITS>(lat, p.nb.d);
+        p.su = spin_get<BITS>(lat, p.nb.u);
+        p.T = minus_ln(r.z, r.w);
+        lead_bracket(p.T, small_k, tsh, 0, p.blo, p.bw);
+    };
+    if (live) {
+    // The current bin's shadow AF and its visits since the walker came are kept
+    // in registers, and written when the walker leaves the bin.
+    int Eo = E_io - lo;
+    long long AF = lgf[REWL_IDX(Eo, 0, M.B, tally.bad)];
+    uint32_t visits = 0;
+    unsigned int nacc = 0;
+    unsigned long long t = t_io;
+    const unsigned long long t_end = t_io + (unsigned long long)M.K;
+    Prop cp;
+    draw(t, cp);
+    for (;;) {
+        const int nw = cp.v + (cp.v >= cp.cur);
+        const int dE = (int)(cp.sr == cp.cur) + (int)(cp.sl == cp.cur) + (int)(cp.sd == cp.cur) + (int)(cp.su == cp.cur) -
+                       (int)(cp.sr == nw) - (int)(cp.sl == nw) - (int)(cp.sd == nw) - (int)(cp.su == nw);
+        const int En = Eo + dE;
+        const long long there = lgf[REWL_IDX(En, -kPad, M.B + kPad, tally.bad)];  // beyond the window: kOutside
+        Prop np;
+        draw(t + 1ull, np);  // (past the last step: drawn, never taken)
+        const long long BF = dE == 0 ? AF : there;
+        const int D = (int)(BF >> 32) - (int)(AF >> 32);
+        bool acc = D < cp.blo;
+        if ((uint32_t)(D - cp.blo) < cp.bw)  // the leading words do not decide
+            acc = decide_1(rare, AF, BF, REWL_IDX(Eo, 0, M.B, tally.bad), REWL_IDX(En, 0, M.B, tally.bad), cp.T, random(t),
+                           &tally.tie, t);
+        const int Eb = acc ? En : Eo;
+        const long long cur = acc ? BF : AF;
+        if (Eb != Eo) {  // leaving the bin: its value and visits go to memory
+            lgf[REWL_IDX(Eo, 0, M.B, tally.bad)] = AF;
+            atomicAdd(&hg[REWL_IDX(Eo, 0, M.B, tally.bad)], visits);  // (result not used: the walker does not wait)
+            visits = 0;
+        }
+        ++visits;
+        Eo = Eb;
+        AF = (long long)((unsigned long long)cur + incF);  // ln g(E) += ln f
+        const uint32_t hc = (uint32_t)((unsigned long long)cur >> 32), h2 = (uint32_t)((unsigned long long)AF >> 32);
+        if (!int_add || (cur & 1) || (h2 ^ hc) > hc) AF = add_1(rare, cur, REWL_IDX(Eb, 0, M.B, tally.bad), AF, int_add);
+        if (acc) {
+            if (BITS == 8) reinterpret_cast<uint8_t *>(lat)[cp.site] = (uint8_t)nw;
+            else atomicXor(&lat[cp.site / per], (uint32_t)(cp.cur ^ nw) << ((cp.site & (per - 1)) * BITS));
+            ++nacc;
+            // the next proposal's spins were read before this flip
+            if (np.site == cp.site) np.cur = nw;
+            if (np.nb.r == cp.site) np.sr = nw;
+            if (np.nb.l == cp.site) np.sl = nw;
+            if (np.nb.d == cp.site) np.sd = nw;
+            if (np.nb.u == cp.site) np.su = nw;
+        }
+        if (++t == t_end) break;
+        cp = np;
+    }
+    lgf[Eo] = AF;
+    atomicAdd(&hg[Eo], visits);
+    t_io = t_end;
+    E_io = Eo + lo;
+    tally.acc += nacc;
+    tally.slow += rare.slow;
+    tally.seq += rare.seq;
+    }
+    __syncwarp();
+    for (unsigned rest = lanes; rest; rest &= rest - 1u) {
+        const int w = __ffs((int)rest) - 1, B = __shfl_sync(0xffffffffu, M.B, w), e = __shfl_sync(0xffffffffu, rare.ew, w);
+        const long long *f = of(lgf, w);
+        long long *v = of(lgb, w);
+        for (int b0 = lane; b0 < B; b0 += 32 * kInFlight) {
+            long long x[kInFlight];
+#pragma unroll
+            for (int i = 0; i < kInFlight; ++i) x[i] = b0 + 32 * i < B ? f[b0 + 32 * i] : 1;
+#pragma unroll
+            for (int i = 0; i < kInFlight; ++i)
+                if (!(x[i] & 1)) v[b0 + 32 * i] = from_units(x[i] >> 1, e);
+        }
+    }
 }
 
 // S > 1 lanes per walker: batches of S steps, lane j owning step j.
@@ -515,10 +609,7 @@ template <int BITS, int S, bool PROD = false>
 __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb,
                                              long long *lgf, uint32_t *__restrict__ hg, const Stage &st, int g, int lo,
                                              double lnf, int &E_io, unsigned long long &t_io, Tally &tally) {
-    if constexpr (S == 1) {
-        walker_sweep_1<BITS>(M, lat, lgb, lgf, hg, g, lo, lnf, E_io, t_io, tally);
-        return;
-    } else {
+    static_assert(S > 1, "walker_sweep_1");
     const int j = (int)(threadIdx.x & (unsigned)(S - 1));
     const unsigned gm = group_mask<S>();
     const unsigned gbase = S == 32 ? 0u : threadIdx.x & 31u & ~(unsigned)(S - 1);
@@ -628,12 +719,7 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     auto sts8 = [](uint32_t a, uint32_t v) { *reinterpret_cast<uint8_t *>(__cvta_shared_to_generic(a)) = (uint8_t)v; };
 
     // The part of a proposal that needs no state: site, neighbours, new value,
-    // T = -ln u in 2^-26 (kTiny: u < 2^-24, only D < 0 is decided by it), and
-    // [blo, blo + bw): the leading-word differences that do not decide.  The
-    // true difference D 2^-32 lies strictly within 1 of the difference of the
-    // leading words, kSlack is far below a leading word's unit, and out of the
-    // window the difference is at least 2^30 - 2, above every T at tsh >= 1.
-    constexpr int kTiny = 0x7fffffff;
+    // T = -ln u and the leading words' bracket of it.
     struct Draw {
         int site, v, T, blo;
         uint32_t bw;
@@ -652,14 +738,7 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         philox_blocks<kAhead>(t, (uint32_t)g, DOM_WL, M.rk, r);
 #pragma unroll
         for (int c = 0; c < kAhead; ++c) {
-            // as accept_bracket, in integers: u from its leading 27 bits and the rest
-            // (relative error below 2^-23), -ln u from lg2.approx (absolute or relative
-            // error at most 2^-22, times ln 2) and rounded to 2^-26: together below
-            // (Lf + 1) 2^-21; the margin is (Lf + 1) 2^-18
-            const float uf = fmaf((float)(r[c].z & ~31u), 0x1p-32f, (float)r[c].w * 0x1p-59f);
-            float l2;
-            asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l2) : "f"(uf));
-            const int T = r[c].z < 256u ? kTiny : __float2int_rn(l2 * -0x1.62e43p+25f);  // below 2^31 for u >= 2^-24
+            const int T = minus_ln(r[c].z, r[c].w);
             st.ring[c * S + j] = make_uint2(__umulhi(r[c].x, (uint32_t)N) | __umulhi(r[c].y, qm1) << 20, (uint32_t)T);
         }
     };
@@ -672,13 +751,7 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         d.nb = nbrs(d.site, L, N, M.divL);
         d.twins = bit;
         if (crowded) d.twins = __match_any_sync(gm, d.site) >> gbase;
-        const int mg = (d.T >> 18) + 260;  // (Lf + 1) 2^-18, rounded up
-        d.blo = ((d.T - mg) >> tsh) - 1 - loose;
-        d.bw = (uint32_t)(((d.T + mg) >> tsh) + 3 + loose - d.blo);
-        if (d.T == kTiny || !small_k) {
-            d.blo = small_k ? -2 : -0x7fffffff;
-            d.bw = 0xfffffff0u;
-        }
+        lead_bracket(d.T, small_k, tsh, loose, d.blo, d.bw);
         return d;
     };
     // the same bracket in half-units, from step t's draw
@@ -996,7 +1069,6 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     tally.seq += nseq;
     tally.acc += nacc;
     E_io = (int)(pcur - pbase) / 8 + lo;
-    }
 }
 
 // P walkers g0 .. g0 + P - 1 of one instance: stage their lattices in shared
@@ -1042,6 +1114,21 @@ __device__ __forceinline__ void unstage_lattice(const Model &M, uint32_t *dst, c
     }
 }
 
+// A walker's state and counters after its launch (one thread per walker).
+__device__ __forceinline__ void end_walker(const Model &M, const State &Sg, int g, uint32_t c, int E, unsigned long long t,
+                                           const Tally &tally) {
+    Sg.cfg_E[c] = E;
+    Sg.t[g] = t;
+    atomicAdd(&Sg.ctl->flips, (unsigned long long)M.K);
+    atomicAdd(&Sg.ctl->accepted, (unsigned long long)tally.acc);
+    if (tally.slow) atomicAdd(&Sg.ctl->slow, tally.slow);
+    flush_ties(Sg, g, tally.tie);
+    if (tally.seq) atomicAdd(&Sg.ctl->seq, (unsigned long long)tally.seq);
+#ifdef REWL_DEBUG_CHECKS
+    if (tally.bad) atomicOr(&Sg.ctl->error, ERR_BOUNDS);
+#endif
+}
+
 template <int BITS, int S, bool LG>
 __device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int g0, int P, const Layout &lay,
                                             unsigned char *smem) {
@@ -1070,7 +1157,20 @@ __device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int
     bool live = grp < P && g < M.G;
     if (live) live = !Sg.done[g / M.m];
     if (S == 32) live = __any_sync(0xffffffffu, live);
-    if (live) {
+    if constexpr (S == 1) {
+        unsigned char *base = smem + (size_t)(live ? grp : 0) * lay.stride;
+        const int gl = live ? g : g0, w = gl / M.m;
+        const uint32_t c = Sg.slot_cfg[gl];
+        int E = Sg.cfg_E[c];
+        unsigned long long t = Sg.t[gl];
+        // with global lattices the shadow is in global memory too
+        walker_sweep_1<BITS>(M, LG ? Sg.spins + (size_t)c * M.wpc : reinterpret_cast<uint32_t *>(base + lay.off_lat),
+                             reinterpret_cast<long long *>(Sg.lng + (size_t)gl * M.B),
+                             LG ? Sg.shadow + (size_t)gl * (M.B + 2 * kPad) + kPad
+                                : reinterpret_cast<long long *>(base + lay.off_lgf) + kPad,
+                             Sg.H + (size_t)gl * M.B, gl, Sg.e_lo[w], Sg.lnf[w], E, t, tally, live);
+        if (live) end_walker(M, Sg, gl, c, E, t, tally);
+    } else if (live) {
         unsigned char *base = smem + (size_t)grp * lay.stride;
         Stage st;
         st.ring = reinterpret_cast<uint2 *>(base + lay.off_ring);
@@ -1083,20 +1183,10 @@ __device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int
         int E = Sg.cfg_E[c];
         unsigned long long t = Sg.t[g];
         uint32_t *lat = LG ? Sg.spins + (size_t)c * M.wpc : reinterpret_cast<uint32_t *>(base + lay.off_lat);
-        // one lane with global lattices: the shadow is in global memory too
-        long long *lgf = (S == 1 && LG) ? Sg.shadow + (size_t)g * (M.B + 2 * kPad) + kPad
-                                        : reinterpret_cast<long long *>(base + lay.off_lgf) + kPad;
+        long long *lgf = reinterpret_cast<long long *>(base + lay.off_lgf) + kPad;
         walker_sweep<BITS, S>(M, lat, reinterpret_cast<long long *>(Sg.lng + (size_t)g * M.B), lgf,
                               Sg.H + (size_t)g * M.B, st, g, Sg.e_lo[w], Sg.lnf[w], E, t, tally);
-        if ((threadIdx.x & (S - 1)) == 0) {
-            Sg.cfg_E[c] = E;
-            Sg.t[g] = t;
-            atomicAdd(&Sg.ctl->flips, (unsigned long long)M.K);
-            atomicAdd(&Sg.ctl->accepted, (unsigned long long)tally.acc);
-            if (tally.slow) atomicAdd(&Sg.ctl->slow, tally.slow);
-            flush_ties(Sg, g, tally.tie);
-            if (tally.seq) atomicAdd(&Sg.ctl->seq, (unsigned long long)tally.seq);
-        }
+        if ((threadIdx.x & (S - 1)) == 0) end_walker(M, Sg, g, c, E, t, tally);
 #ifdef REWL_DEBUG_CHECKS
         if (tally.bad) atomicOr(&Sg.ctl->error, ERR_BOUNDS);
 #endif
@@ -1208,34 +1298,19 @@ __global__ void __launch_bounds__(256) batch_sweep_kernel(const InstDev *inst, c
 template <int BITS>
 __global__ void __launch_bounds__(256) batch_walker_kernel(const InstDev *inst, const WalkerItem *items, int n_items) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_items) return;
-    const WalkerItem it = items[i];
-    const Model &M = inst[it.inst].M;
-    const State &Sg = inst[it.inst].S;
-    if (*(volatile unsigned int *)&Sg.ctl->all_done) return;
-    const int g = it.g;
-    if (Sg.done[g / M.m]) return;
-    const Model Mr = M;
-    const State Sr = Sg;
-    Stage st{};
+    const WalkerItem it = items[min(i, n_items - 1)];
+    const Model M = inst[it.inst].M;
+    const State Sg = inst[it.inst].S;
+    const int g = it.g, w = g / M.m;
+    const bool live = i < n_items && !*(volatile unsigned int *)&Sg.ctl->all_done && !Sg.done[w];
     Tally tally{};
-    const int w = g / Mr.m;
-    const uint32_t c = Sr.slot_cfg[g];
-    int E = Sr.cfg_E[c];
-    unsigned long long t = Sr.t[g];
-    walker_sweep<BITS, 1>(Mr, Sr.spins + (size_t)c * Mr.wpc, reinterpret_cast<long long *>(Sr.lng + (size_t)g * Mr.B),
-                          Sr.shadow + (size_t)g * (Mr.B + 2 * kPad) + kPad, Sr.H + (size_t)g * Mr.B, st, g, Sr.e_lo[w],
-                          Sr.lnf[w], E, t, tally);
-    Sr.cfg_E[c] = E;
-    Sr.t[g] = t;
-    atomicAdd(&Sr.ctl->flips, (unsigned long long)Mr.K);
-    atomicAdd(&Sr.ctl->accepted, (unsigned long long)tally.acc);
-    if (tally.slow) atomicAdd(&Sr.ctl->slow, tally.slow);
-    flush_ties(Sr, g, tally.tie);
-    if (tally.seq) atomicAdd(&Sr.ctl->seq, (unsigned long long)tally.seq);
-#ifdef REWL_DEBUG_CHECKS
-    if (tally.bad) atomicOr(&Sr.ctl->error, ERR_BOUNDS);
-#endif
+    const uint32_t c = Sg.slot_cfg[g];
+    int E = Sg.cfg_E[c];
+    unsigned long long t = Sg.t[g];
+    walker_sweep_1<BITS>(M, Sg.spins + (size_t)c * M.wpc, reinterpret_cast<long long *>(Sg.lng + (size_t)g * M.B),
+                         Sg.shadow + (size_t)g * (M.B + 2 * kPad) + kPad, Sg.H + (size_t)g * M.B, g, Sg.e_lo[w],
+                         Sg.lnf[w], E, t, tally, live);
+    if (live) end_walker(M, Sg, g, c, E, t, tally);
 }
 
 // Bits per spin of a lattice staged in shared memory: bytes, one load per spin
