@@ -347,9 +347,9 @@ __device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, i
 // stores to the lattice (the thread owns it) and the current bin's shadow and
 // visits in registers until the walker leaves the bin.  The passes over all bins
 // before and after the steps are taken by the warp together, one walker after
-// another, so that the lanes' loads lie side by side (3.1 -> @W2@ ms on 2048
+// another, so that the lanes' loads lie side by side (3.1 -> 1.0 ms on 2048
 // instances).  Every thread of a warp calls, live or not.  2048 instances, 56,784
-// walkers, 10^4 steps: 16.1 -> @W1@ ms a round.
+// walkers, 10^4 steps: 16.1 -> 9.7 ms a round.
 struct Slow1 {  // what the rare parts of a step need
     long long *lgb;
     double lnf;
@@ -385,7 +385,7 @@ __device__ __noinline__ long long add_1(Slow1 &s, long long F, int b, long long 
 
 constexpr int kInFlight = 8;  // loads of such a pass in flight per lane
 
-template <int BITS>
+template <int BITS, bool GLOBAL>
 __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb, long long *lgf,
                                uint32_t *__restrict__ hg, int g, int lo, double lnf, int &E_io,
                                unsigned long long &t_io, Tally &tally, bool live) {
@@ -393,6 +393,12 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
     constexpr int per = 32 / BITS;
     const uint32_t qm1 = (uint32_t)(M.q - 1), divL = M.divL;
     const long long LNF = __double_as_longlong(lnf);
+    if (GLOBAL) {
+        __builtin_assume(__isGlobal(lat));
+        __builtin_assume(__isGlobal(lgf));
+    }
+    __builtin_assume(__isGlobal(lgb));
+    __builtin_assume(__isGlobal(hg));
     const int lane = (int)(threadIdx.x & 31u);
     const unsigned lanes = __ballot_sync(0xffffffffu, live);
     auto of = [&](auto *p, int w) {  // lane w's pointer
@@ -402,6 +408,7 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
     for (unsigned rest = lanes; rest; rest &= rest - 1u) {
         const int w = __ffs((int)rest) - 1, B = __shfl_sync(0xffffffffu, M.B, w);
         const long long *v = of(lgb, w);
+        __builtin_assume(__isGlobal(v));
         long long top = 0;
         for (int b0 = lane; b0 < B; b0 += 32 * kInFlight) {
             long long x[kInFlight];
@@ -427,6 +434,8 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         const int w = __ffs((int)rest) - 1, B = __shfl_sync(0xffffffffu, M.B, w), e = __shfl_sync(0xffffffffu, rare.ew, w);
         const long long *v = of(lgb, w);
         long long *f = of(lgf, w);
+        __builtin_assume(__isGlobal(v));
+        if (GLOBAL) __builtin_assume(__isGlobal(f));
         for (int b0 = lane; b0 < B; b0 += 32 * kInFlight) {
             long long x[kInFlight];
 #pragma unroll
@@ -451,6 +460,8 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         rk[2 * r] = M.key0 + r * 0x9E3779B9u;
         rk[2 * r + 1] = M.key1 + r * 0xBB67AE85u;
     }
+#pragma unroll
+    for (int r = 0; r < 20; ++r) asm("" : "+r"(rk[r]));  // kept, not added up again in every block
 
     struct Prop {
         int site, v, cur, sr, sl, sd, su, T, blo;
@@ -482,16 +493,22 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
     unsigned int nacc = 0;
     unsigned long long t = t_io;
     const unsigned long long t_end = t_io + (unsigned long long)M.K;
-    Prop cp;
-    draw(t, cp);
-    for (;;) {
+    // Two proposals wait with their spins read, so that a step's reads have two
+    // steps to arrive; both take over a flip in registers.
+    auto flipped = [](Prop &p, int site, int to) {
+        if (p.site == site) p.cur = to;
+        if (p.nb.r == site) p.sr = to;
+        if (p.nb.l == site) p.sl = to;
+        if (p.nb.d == site) p.sd = to;
+        if (p.nb.u == site) p.su = to;
+    };
+    auto step = [&](const Prop &cp, Prop &n1, Prop &n2) {
         const int nw = cp.v + (cp.v >= cp.cur);
         const int dE = (int)(cp.sr == cp.cur) + (int)(cp.sl == cp.cur) + (int)(cp.sd == cp.cur) + (int)(cp.su == cp.cur) -
                        (int)(cp.sr == nw) - (int)(cp.sl == nw) - (int)(cp.sd == nw) - (int)(cp.su == nw);
         const int En = Eo + dE;
         const long long there = lgf[REWL_IDX(En, -kPad, M.B + kPad, tally.bad)];  // beyond the window: kOutside
-        Prop np;
-        draw(t + 1ull, np);  // (past the last step: drawn, never taken)
+        draw(t + 2ull, n2);  // (past the last step: drawn, never taken)
         const long long BF = dE == 0 ? AF : there;
         const int D = (int)(BF >> 32) - (int)(AF >> 32);
         bool acc = D < cp.blo;
@@ -509,20 +526,24 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         Eo = Eb;
         AF = (long long)((unsigned long long)cur + incF);  // ln g(E) += ln f
         const uint32_t hc = (uint32_t)((unsigned long long)cur >> 32), h2 = (uint32_t)((unsigned long long)AF >> 32);
-        if (!int_add || (cur & 1) || (h2 ^ hc) > hc) AF = add_1(rare, cur, REWL_IDX(Eb, 0, M.B, tally.bad), AF, int_add);
+        if (!int_add || (cur & 1) || (h2 ^ hc) > hc) {
+            const int sh = 11 - __clzll(AF >> 1);  // (whole_steps, its usual case)
+            if (!int_add || (cur & 1) || (sh > 0 && ((AF >> 1) & ((1LL << sh) - 1)) != 0))
+                AF = add_1(rare, cur, REWL_IDX(Eb, 0, M.B, tally.bad), AF, int_add);
+        }
         if (acc) {
             if (BITS == 8) reinterpret_cast<uint8_t *>(lat)[cp.site] = (uint8_t)nw;
             else atomicXor(&lat[cp.site / per], (uint32_t)(cp.cur ^ nw) << ((cp.site & (per - 1)) * BITS));
             ++nacc;
-            // the next proposal's spins were read before this flip
-            if (np.site == cp.site) np.cur = nw;
-            if (np.nb.r == cp.site) np.sr = nw;
-            if (np.nb.l == cp.site) np.sl = nw;
-            if (np.nb.d == cp.site) np.sd = nw;
-            if (np.nb.u == cp.site) np.su = nw;
+            flipped(n1, cp.site, nw);
+            flipped(n2, cp.site, nw);
         }
-        if (++t == t_end) break;
-        cp = np;
+        return ++t == t_end;
+    };
+    Prop a, b, c;
+    draw(t, a);
+    draw(t + 1ull, b);
+    while (!step(a, b, c) && !step(b, c, a) && !step(c, a, b)) {
     }
     lgf[Eo] = AF;
     atomicAdd(&hg[Eo], visits);
@@ -537,6 +558,8 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         const int w = __ffs((int)rest) - 1, B = __shfl_sync(0xffffffffu, M.B, w), e = __shfl_sync(0xffffffffu, rare.ew, w);
         const long long *f = of(lgf, w);
         long long *v = of(lgb, w);
+        __builtin_assume(__isGlobal(v));
+        if (GLOBAL) __builtin_assume(__isGlobal(f));
         for (int b0 = lane; b0 < B; b0 += 32 * kInFlight) {
             long long x[kInFlight];
 #pragma unroll
@@ -1164,7 +1187,7 @@ __device__ __forceinline__ void sweep_block(const Model &M, const State &Sg, int
         int E = Sg.cfg_E[c];
         unsigned long long t = Sg.t[gl];
         // with global lattices the shadow is in global memory too
-        walker_sweep_1<BITS>(M, LG ? Sg.spins + (size_t)c * M.wpc : reinterpret_cast<uint32_t *>(base + lay.off_lat),
+        walker_sweep_1<BITS, LG>(M, LG ? Sg.spins + (size_t)c * M.wpc : reinterpret_cast<uint32_t *>(base + lay.off_lat),
                              reinterpret_cast<long long *>(Sg.lng + (size_t)gl * M.B),
                              LG ? Sg.shadow + (size_t)gl * (M.B + 2 * kPad) + kPad
                                 : reinterpret_cast<long long *>(base + lay.off_lgf) + kPad,
@@ -1307,7 +1330,7 @@ __global__ void __launch_bounds__(256) batch_walker_kernel(const InstDev *inst, 
     const uint32_t c = Sg.slot_cfg[g];
     int E = Sg.cfg_E[c];
     unsigned long long t = Sg.t[g];
-    walker_sweep_1<BITS>(M, Sg.spins + (size_t)c * M.wpc, reinterpret_cast<long long *>(Sg.lng + (size_t)g * M.B),
+    walker_sweep_1<BITS, true>(M, Sg.spins + (size_t)c * M.wpc, reinterpret_cast<long long *>(Sg.lng + (size_t)g * M.B),
                          Sg.shadow + (size_t)g * (M.B + 2 * kPad) + kPad, Sg.H + (size_t)g * M.B, g, Sg.e_lo[w],
                          Sg.lnf[w], E, t, tally, live);
     if (live) end_walker(M, Sg, g, c, E, t, tally);
