@@ -382,72 +382,135 @@ __global__ void count_spins_kernel(Model M, State S) {
 constexpr int MAX_M = 256;  // walkers per window (exchange permutation buffer)
 constexpr int CHECK_THREADS = 256;
 
+// Whether walkers 0 .. m - 1 of a window are all flat over its mask, which takes
+// in the bins they visited; n_bins: bins in the mask; ovf: a bin at 2^31 visits.
+// At most MM walkers: one pass over the bins, every walker's sums in registers.
+// (q = 10, L = 80, 64 windows of 16: 27 -> 13 us; 19,113 windows of 2 or 4: 223 ->
+// 165 us, against a pass per walker with two barriers each.)
+template <int MM>
+__device__ __forceinline__ bool flat_in_one_pass(const Model &M, const uint32_t *H, uint8_t *mask, bool inv_t,
+                                                 unsigned int &n_bins, int &ovf) {
+    constexpr int NW = CHECK_THREADS / 32;
+    __shared__ unsigned int p_n[NW], p_mn[NW][MM], p_any[NW];
+    __shared__ unsigned long long p_sum[NW][MM];
+    const int B = M.B, m = M.m, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    unsigned int n = 0, mn[MM], top = 0;
+    unsigned long long sum[MM];
+#pragma unroll
+    for (int k = 0; k < MM; ++k) {
+        mn[k] = 0xffffffffu;
+        sum[k] = 0;
+    }
+    for (int b = tid; b < B; b += CHECK_THREADS) {
+        uint32_t hv[MM], any = 0;
+#pragma unroll
+        for (int k = 0; k < MM; ++k) {
+            hv[k] = k < m ? H[(size_t)k * B + b] : 0u;
+            any |= hv[k];
+        }
+        const uint8_t was = mask[b];
+        if (any && !was) mask[b] = 1;
+        top |= any;  // (the top bit)
+        if (!any && !was) continue;
+        n += 1u;
+#pragma unroll
+        for (int k = 0; k < MM; ++k) {
+            sum[k] += hv[k];
+            mn[k] = min(mn[k], hv[k]);
+        }
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    top = __reduce_or_sync(0xffffffffu, top);
+#pragma unroll
+    for (int k = 0; k < MM; ++k) {
+        mn[k] = __reduce_min_sync(0xffffffffu, mn[k]);
+        for (int o = 16; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], o);
+    }
+    if (lane == 0) {
+        p_n[wid] = n;
+        p_any[wid] = top;
+#pragma unroll
+        for (int k = 0; k < MM; ++k) {
+            p_mn[wid][k] = mn[k];
+            p_sum[wid][k] = sum[k];
+        }
+    }
+    __syncthreads();
+    n = 0;
+    top = 0;
+    for (int i = 0; i < NW; ++i) {
+        n += p_n[i];
+        top |= p_any[i];
+    }
+    bool flat = true;
+    if (tid < m) {
+        unsigned int least = 0xffffffffu;
+        unsigned long long all = 0;
+        for (int i = 0; i < NW; ++i) {
+            least = min(least, p_mn[i][tid]);
+            all += p_sum[i][tid];
+        }
+        flat = n > 0 && (inv_t ? least >= 1u : (double)least >= M.flatness * ((double)all / (double)n));
+    }
+    n_bins = n;
+    ovf = top >= 0x80000000u;
+    return __syncthreads_and(flat);
+}
+
+// Any number of walkers: the mask first, then a warp per walker.
+__device__ __forceinline__ bool flat_by_walkers(const Model &M, const uint32_t *H, uint8_t *mask, bool inv_t,
+                                                unsigned int &n_bins, int &ovf) {
+    __shared__ unsigned int s_bins;
+    const int B = M.B, m = M.m, tid = threadIdx.x, lane = tid & 31;
+    int over = 0;
+    for (int b = tid; b < B; b += CHECK_THREADS) {
+        uint32_t any = 0;  // (the top bit: a bin at 2^31 visits)
+#pragma unroll 8
+        for (int k = 0; k < m; ++k) any |= H[(size_t)k * B + b];
+        over |= any >= 0x80000000u;
+        if (any) mask[b] = 1;
+    }
+    ovf = __syncthreads_or(over);
+    bool flat = true;
+    for (int k = tid >> 5; k < m; k += CHECK_THREADS / 32) {
+        unsigned int n = 0, mn = 0xffffffffu;
+        unsigned long long sum = 0;
+        const uint32_t *hk = H + (size_t)k * B;
+#pragma unroll 4
+        for (int b = lane; b < B; b += 32) {
+            const uint32_t hv = hk[b];
+            if (!mask[b]) continue;
+            n += 1u;
+            sum += hv;
+            mn = min(mn, hv);
+        }
+        n = __reduce_add_sync(0xffffffffu, n);
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        flat = flat && n > 0 && (inv_t ? mn >= 1u : (double)mn >= M.flatness * ((double)sum / (double)n));
+        if (tid == 0 && k == 0) s_bins = n;  // (the mask is the window's: any walker's count)
+    }
+    const bool all = __syncthreads_and(flat);
+    n_bins = s_bins;
+    return all;
+}
+
 __device__ void window_check_block(const Model &M, const State &S, int w) {
     if (*(volatile unsigned int *)&S.ctl->all_done) return;
     if (S.done[w]) return;
     const int B = M.B, m = M.m, tid = threadIdx.x;
     const size_t base = (size_t)w * m * B;
     uint8_t *mask = S.mask + (size_t)w * B;
-
-    int ovf = 0;
-    for (int b = tid; b < B; b += blockDim.x) {
-        int vis = 0;
-        for (int k = 0; k < m; ++k) {
-            const uint32_t hv = S.H[base + (size_t)k * B + b];
-            vis |= hv > 0u;
-            ovf |= hv >= 0x80000000u;
-        }
-        if (vis) mask[b] = 1;
-    }
-    if (__syncthreads_or(ovf)) {
+    const bool inv_t = M.schedule == SCHED_INV_T;
+    const bool follows_1t = inv_t && S.phase[w];
+    unsigned int n_bins;
+    int ovf;
+    const bool all_flat = m <= 4 ? flat_in_one_pass<4>(M, S.H + base, mask, inv_t, n_bins, ovf)
+                                 : flat_by_walkers(M, S.H + base, mask, inv_t, n_bins, ovf);
+    if (ovf) {
         if (tid == 0) atomicOr(&S.ctl->error, ERR_OVERFLOW);
         return;
     }
-
-    const bool inv_t = M.schedule == SCHED_INV_T;
-    const bool follows_1t = inv_t && S.phase[w];
-    __shared__ unsigned int r_n[CHECK_THREADS / 32], r_mn[CHECK_THREADS / 32];
-    __shared__ unsigned long long r_sum[CHECK_THREADS / 32];
-    __shared__ int all_flat;
-    __shared__ unsigned int n_bins;  // bins in the window's mask
-    if (tid == 0) all_flat = 1;
-    for (int k = 0; k < m; ++k) {
-        unsigned int n = 0, mn = 0xffffffffu;
-        unsigned long long sum = 0;
-        const uint32_t *hk = S.H + base + (size_t)k * B;
-        for (int b = tid; b < B; b += blockDim.x) {
-            if (!mask[b]) continue;
-            const uint32_t hv = hk[b];
-            n += 1u;
-            sum += hv;
-            mn = min(mn, hv);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            n += __shfl_xor_sync(0xffffffffu, n, o);
-            sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        }
-        __syncthreads();
-        if ((tid & 31) == 0) {
-            r_n[tid >> 5] = n;
-            r_sum[tid >> 5] = sum;
-            r_mn[tid >> 5] = mn;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            unsigned int tn = 0, tmn = 0xffffffffu;
-            unsigned long long ts = 0;
-            for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-                tn += r_n[i];
-                ts += r_sum[i];
-                tmn = min(tmn, r_mn[i]);
-            }
-            const bool flat = tn > 0 && (inv_t ? tmn >= 1u : (double)tmn >= M.flatness * ((double)ts / (double)tn));
-            if (!flat) all_flat = 0;
-            n_bins = tn;
-        }
-    }
-    __syncthreads();
     if (!all_flat && !follows_1t) return;
 
     // Merge: the pairwise tree is formed in place in the walkers' own rows (they
@@ -500,24 +563,39 @@ __global__ void __launch_bounds__(CHECK_THREADS) window_check_kernel(Model M, St
 // configurations with probability min[1, g_i(E_X) g_j(E_Y) / (g_i(E_Y) g_j(E_X))].
 // A swap exchanges the two walkers' buffer ids; ln g and H stay with the walkers.
 // Then the round counter advances and the completion flag is refreshed.
+//
+// What bounds it: a chain of dependent loads (buffer ids, energies, ln g) in a
+// single CTA.  So a thread shuffles the partners of one pair of windows and a
+// thread decides one pair of walkers, as many at a time as the shared table of
+// partners holds, and the chain is walked once: q = 10, L = 300, 717 windows of
+// 3: 59 -> 16 us (a warp per pair of windows walked it twelve times).
 constexpr int XCH_THREADS = 1024;
+constexpr int XCH_PARTNERS = 8192;  // walkers matched at a time
+// Batches: a small CTA per instance (2048 instances: 73 -> 18 us).
+constexpr int XCH_BATCH_THREADS = 128, XCH_BATCH_PARTNERS = 1024;
 
+template <int PARTNERS>
 __device__ void exchange_block(const Model &M, const State &S) {
-    __shared__ int perm[XCH_THREADS / 32][MAX_M];
+    static_assert(PARTNERS >= MAX_M, "one pair of windows at least");
+    __shared__ int perm[PARTNERS];
     Ctl *ctl = S.ctl;
     if (!M.production && *(volatile unsigned int *)&ctl->all_done) return;
     const unsigned long long round = ctl->round;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    const int m = M.m, B = M.B;
+    const int m = M.m, B = M.B, first = (int)(round & 1ull);
+    const int pairs = M.h > first ? (M.h - first) / 2 : 0;  // windows (first + 2 p, first + 2 p + 1)
+    const int at_once = PARTNERS / m;                       // m <= MAX_M
     unsigned long long tried = 0, acc = 0;
-    for (int a = (int)(round & 1ull) + 2 * warp; a + 1 < M.h; a += 2 * nwarps) {
-        if (!M.production && (S.done[a] || S.done[a + 1])) continue;  // production: every pair
-        int *pi = perm[warp];
-        if (lane == 0) {
+    for (int p0 = 0; p0 < pairs; p0 += at_once) {
+        const int np = min(at_once, pairs - p0);
+        for (int p = (int)threadIdx.x; p < np; p += (int)blockDim.x) {
+            const int a = first + 2 * (p0 + p);
+            if (!M.production && (S.done[a] || S.done[a + 1])) continue;  // production: every pair
+            int *pi = perm + p * m;
             for (int k = 0; k < m; ++k) pi[k] = k;
+            uint4 r = make_uint4(0u, 0u, 0u, 0u);
             for (int i = m - 1; i >= 1; --i) {
                 const int n = m - 1 - i;
-                const uint4 r = philox((uint32_t)round, (uint32_t)(n >> 2), (uint32_t)a, DOM_PERM, M.key0, M.key1);
+                if ((n & 3) == 0) r = philox((uint32_t)round, (uint32_t)(n >> 2), (uint32_t)a, DOM_PERM, M.key0, M.key1);
                 const uint32_t word = (n & 3) == 0 ? r.x : (n & 3) == 1 ? r.y : (n & 3) == 2 ? r.z : r.w;
                 const int j = (int)__umulhi(word, (uint32_t)(i + 1));
                 const int tmp = pi[i];
@@ -525,11 +603,13 @@ __device__ void exchange_block(const Model &M, const State &S) {
                 pi[j] = tmp;
             }
         }
-        __syncwarp();
-        const int lo_a = S.e_lo[a], hi_a = lo_a + M.W;
-        const int lo_b = S.e_lo[a + 1], hi_b = lo_b + M.W;
-        for (int k = lane; k < m; k += 32) {
-            const int gi = a * m + k, gj = (a + 1) * m + pi[k];
+        __syncthreads();
+        for (int x = (int)threadIdx.x; x < np * m; x += (int)blockDim.x) {
+            const int p = x / m, k = x - p * m, a = first + 2 * (p0 + p);
+            if (!M.production && (S.done[a] || S.done[a + 1])) continue;
+            const int lo_a = S.e_lo[a], hi_a = lo_a + M.W;
+            const int lo_b = S.e_lo[a + 1], hi_b = lo_b + M.W;
+            const int gi = a * m + k, gj = (a + 1) * m + perm[x];
             const uint32_t ci = S.slot_cfg[gi], cj = S.slot_cfg[gj];
             const int Ei = S.cfg_E[ci], Ej = S.cfg_E[cj];
             if (!(Ei >= lo_b && Ei <= hi_b && Ej >= lo_a && Ej <= hi_a)) continue;
@@ -550,7 +630,7 @@ __device__ void exchange_block(const Model &M, const State &S) {
                 ++acc;
             }
         }
-        __syncwarp();
+        __syncthreads();
     }
     if (tried) atomicAdd(&ctl->xtried, tried);
     if (acc) atomicAdd(&ctl->xacc, acc);
@@ -569,15 +649,18 @@ __device__ void exchange_block(const Model &M, const State &S) {
             }
         }
     }
+    int all = 1;
+    for (int w = (int)threadIdx.x; w < M.h; w += (int)blockDim.x) all &= S.done[w] != 0;
+    all = __syncthreads_and(all);
     if (threadIdx.x == 0) {
         ctl->round = round + 1ull;
-        unsigned int all = 1u;
-        for (int w = 0; w < M.h; ++w) all &= (unsigned int)(S.done[w] != 0);
-        ctl->all_done = all;
+        ctl->all_done = (unsigned int)all;
     }
 }
 
-__global__ void __launch_bounds__(XCH_THREADS) exchange_kernel(Model M, State S) { exchange_block(M, S); }
+__global__ void __launch_bounds__(XCH_THREADS) exchange_kernel(Model M, State S) {
+    exchange_block<XCH_PARTNERS>(M, S);
+}
 
 // ---------------------------------------------------------------------------
 // Batched forms: many independent instances in one launch.  Every CTA looks up
@@ -589,10 +672,10 @@ __global__ void __launch_bounds__(CHECK_THREADS) batch_check_kernel(const InstDe
     window_check_block(M, S, it.w);
 }
 
-__global__ void __launch_bounds__(XCH_THREADS) batch_exchange_kernel(const InstDev *inst) {
+__global__ void __launch_bounds__(XCH_BATCH_THREADS) batch_exchange_kernel(const InstDev *inst) {
     const Model M = inst[blockIdx.x].M;
     const State S = inst[blockIdx.x].S;
-    exchange_block(M, S);
+    exchange_block<XCH_BATCH_PARTNERS>(M, S);
 }
 
 // ---------------------------------------------------------------------------
@@ -759,7 +842,7 @@ cudaError_t launch_batch_check(const InstDev *inst, const WinItem *wins, int n_w
 
 cudaError_t launch_batch_exchange(const InstDev *inst, int n_inst, cudaStream_t s) {
     if (n_inst <= 0) return cudaSuccess;
-    batch_exchange_kernel<<<n_inst, XCH_THREADS, 0, s>>>(inst);
+    batch_exchange_kernel<<<n_inst, XCH_BATCH_THREADS, 0, s>>>(inst);
     return cudaGetLastError();
 }
 
