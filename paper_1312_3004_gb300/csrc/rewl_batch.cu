@@ -22,6 +22,12 @@ using rewl::host::fail;
 namespace {
 
 constexpr int kBatchGraphRounds = 4;
+constexpr int kSideStreams = 7;
+// Walkers of a sweep CTA in lane groups: a quarter of what fits its shared memory
+// (and the most a CTA can hold).  A CTA ends with its slowest walker, and small
+// CTAs fill an SM's shared memory: 64 instances (1775 walkers) 1.42 -> @B64@ ms a
+// round, 512 instances 6.9 -> @B512@ ms.
+constexpr int kCtaShare = 4;
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -40,8 +46,12 @@ struct Config {
     int threads = 32;       // lanes 1: threads per CTA (a warp: 1775 of them spread evenly over 152 SMs)
 };
 
+// One sweep launch: walkers of one packing and, in lane groups, of similar
+// shared memory, so that a small walker does not hold a large one's share (the
+// launches of a round run side by side, see enqueue_batch_round).
 struct SweepClass {
     int bits = 4, lanes = 32, threads = 0, grid = 0;
+    size_t most = 0;  // lane groups: bytes per walker, at most
     size_t smem = 0;
     std::vector<rewl::SweepItem> items;      // lanes 32: groups of walkers of one instance
     rewl::SweepItem *d_items = nullptr;
@@ -68,6 +78,8 @@ struct rewl_batch_s {
     rewl::Ctl *h_ctls = nullptr;  // pinned mirrors of every instance's control block
     rewl::Ctl *d_ctls = nullptr;  // the control blocks, contiguous
     cudaStream_t own_stream = nullptr, stream = nullptr;
+    cudaStream_t side[kSideStreams] = {};  // for the round's other sweep launches
+    cudaEvent_t forked = nullptr, joined[kSideStreams] = {};
     // tables of the current configuration (rebuilt by configure)
     rewl::host::DevBlock tblock;
     rewl::InstDev *d_inst = nullptr;
@@ -88,13 +100,26 @@ namespace {
 
 rewl_status enqueue_batch_round(rewl_batch_s *b, cudaStream_t s) {
     BATCH_CUDA(cudaMemsetAsync(b->d_queues, 0, sizeof(unsigned int) * b->classes.size(), s));
-    for (auto &c : b->classes) {
+    // the sweep launches side by side: the first on s, the others on streams that
+    // start behind s and that s waits for
+    const int sides = std::min((int)b->classes.size() - 1, kSideStreams);
+    if (sides > 0) {
+        BATCH_CUDA(cudaEventRecord(b->forked, s));
+        for (int i = 0; i < sides; ++i) BATCH_CUDA(cudaStreamWaitEvent(b->side[i], b->forked, 0));
+    }
+    for (size_t k = 0; k < b->classes.size(); ++k) {
+        SweepClass &c = b->classes[k];
+        const cudaStream_t to = k == 0 ? s : b->side[(k - 1) % kSideStreams];
         if (c.lanes == 1)
             BATCH_CUDA(rewl::launch_batch_walkers(c.bits, b->d_inst, c.d_walkers, (int)c.walkers.size(), c.grid,
-                                                  c.threads, s, false));
+                                                  c.threads, to, false));
         else
             BATCH_CUDA(rewl::launch_batch_sweep(c.bits, c.lanes, b->d_inst, c.d_items, (int)c.items.size(), c.d_queue,
-                                                c.grid, c.threads, c.smem, s, false));
+                                                c.grid, c.threads, c.smem, to, false));
+    }
+    for (int i = 0; i < sides; ++i) {
+        BATCH_CUDA(cudaEventRecord(b->joined[i], b->side[i]));
+        BATCH_CUDA(cudaStreamWaitEvent(s, b->joined[i], 0));
     }
     BATCH_CUDA(rewl::launch_batch_check(b->d_inst, b->d_wins, b->n_wins, s));
     BATCH_CUDA(rewl::launch_batch_exchange(b->d_inst, (int)b->inst.size(), s));
@@ -154,6 +179,11 @@ void destroy_batch(rewl_batch_s *b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->graph) cudaGraphExecDestroy(b->graph);
     for (rewl_s *h : b->inst) delete h;
+    for (cudaStream_t x : b->side)
+        if (x) cudaStreamDestroy(x);
+    for (cudaEvent_t x : b->joined)
+        if (x) cudaEventDestroy(x);
+    if (b->forked) cudaEventDestroy(b->forked);
     if (b->own_stream) cudaStreamDestroy(b->own_stream);
     if (b->h_ctls) cudaFreeHost(b->h_ctls);
     rewl::host::dev_free(b->tblock);
@@ -215,13 +245,18 @@ rewl_status configure(rewl_batch_s *b, const Config &c) {
         tab[(size_t)i].S = h->S;
         tab[(size_t)i].lay = rewl::fast_layout(h->M, c.lanes, c.lanes == 1);
         const int bits = rewl::sweep_bits(h->M, c.lanes, c.lanes == 1);
+        const rewl::Layout &lay = tab[(size_t)i].lay;
+        size_t most = 0;  // classes of bytes per walker in steps of 1.4
+        if (c.lanes != 1)
+            for (most = 4096; most < (size_t)lay.stride;) most = most * 7 / 5;
         int cls = -1;
         for (size_t k = 0; k < b->classes.size(); ++k)
-            if (b->classes[k].bits == bits) cls = (int)k;
+            if (b->classes[k].bits == bits && b->classes[k].most == most) cls = (int)k;
         if (cls < 0) {
             SweepClass sc;
             sc.bits = bits;
             sc.lanes = c.lanes;
+            sc.most = most;
             b->classes.push_back(sc);
             cls = (int)b->classes.size() - 1;
         }
@@ -230,13 +265,14 @@ rewl_status configure(rewl_batch_s *b, const Config &c) {
             for (int g = 0; g < h->M.G; ++g) sc.walkers.push_back({i, g});
             continue;
         }
-        const rewl::Layout &lay = tab[(size_t)i].lay;
         int P = (int)(std::max(budget, (size_t)lay.stride) / (size_t)lay.stride);
-        P = std::min(P, 256 / sc.lanes);
+        P = std::max(1, std::min(P, 256 / sc.lanes) / kCtaShare);
         for (int g0 = 0; g0 < h->M.G; g0 += P) sc.items.push_back({i, g0, std::min(P, h->M.G - g0), 0});
         sc.smem = std::max(sc.smem, (size_t)P * (size_t)lay.stride);
         sc.threads = std::max(sc.threads, P * sc.lanes);
     }
+    // large walkers first: the small ones fill what they leave
+    std::sort(b->classes.begin(), b->classes.end(), [](const SweepClass &x, const SweepClass &y) { return x.most > y.most; });
     size_t off = 0;
     const size_t off_tab = off;
     off += align256((size_t)n * sizeof(rewl::InstDev));
@@ -356,6 +392,12 @@ rewl_status rewl_batch_create_ext(const rewl_params *jobs, int n, int spin_bits,
     e = cudaStreamCreateWithFlags(&b->own_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cleanup(fail(REWL_ERR_CUDA, "stream: %s", cudaGetErrorString(e)));
     b->stream = b->own_stream;
+    e = cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming);
+    for (int i = 0; i < kSideStreams && e == cudaSuccess; ++i) {
+        e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->joined[i], cudaEventDisableTiming);
+    }
+    if (e != cudaSuccess) return cleanup(fail(REWL_ERR_CUDA, "streams: %s", cudaGetErrorString(e)));
     e = cudaMallocHost(&b->h_ctls, (size_t)n * sizeof(rewl::Ctl));
     if (e != cudaSuccess) return cleanup(fail(REWL_ERR_NOMEM, "cudaMallocHost: %s", cudaGetErrorString(e)));
     char *base = (char *)b->dmem;

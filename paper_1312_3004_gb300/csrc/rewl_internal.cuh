@@ -161,6 +161,10 @@ cudaError_t launch_init(const Model &M, const State &S, cudaStream_t s);
 SweepPlan plan_sweep(const Model &M, int num_sms, size_t smem_optin, int kind = SWEEP_FAST, int lanes = 0,
                      int lat_mode = 0);
 cudaError_t prepare_sweep(const Model &M, const SweepPlan &p);
+// Let a kernel take all the shared memory a CTA can have.  (One limit per kernel
+// for the whole process: a handle, batch or server that set it to its own need
+// would take it from those with larger walkers.)
+cudaError_t allow_shared(const void *kernel);
 cudaError_t launch_sweep(const Model &M, const State &S, const SweepPlan &p, cudaStream_t s);
 cudaError_t launch_window_check(const Model &M, const State &S, cudaStream_t s);
 cudaError_t launch_exchange(const Model &M, const State &S, cudaStream_t s);

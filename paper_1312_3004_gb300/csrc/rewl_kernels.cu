@@ -773,6 +773,18 @@ __global__ void energy_check_kernel(Model M, State S) {
 #endif
 
 // ---------------------------------------------------------------------------
+cudaError_t allow_shared(const void *kernel) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    const int most = optin - (int)a.sharedSizeBytes;
+    if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 size_t sweep_smem_per_walker(const Model &M) {
     return (size_t)M.B * (sizeof(double) + sizeof(uint32_t)) + (size_t)M.wpc * sizeof(uint32_t);
 }
@@ -836,9 +848,7 @@ cudaError_t launch_init(const Model &M, const State &S, cudaStream_t s) {
 
 cudaError_t prepare_sweep(const Model &M, const SweepPlan &p) {
     if (p.kind == SWEEP_FAST) return launch_sweep_fast(M, State{}, p, nullptr, true);
-    if (M.bits == 8)
-        return cudaFuncSetAttribute(sweep_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-    return cudaFuncSetAttribute(sweep_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    return allow_shared(M.bits == 8 ? (const void *)sweep_kernel<8> : (const void *)sweep_kernel<4>);
 }
 
 cudaError_t launch_sweep(const Model &M, const State &S, const SweepPlan &p, cudaStream_t s) {

@@ -166,6 +166,11 @@ rewl_status rebuild_tables(rewl_server_s *s) {
         c.threads = 32;
         c.smem = 0;
     }
+    // walkers of a sweep CTA: few enough to spread over the SMs (each is one chain
+    // of steps, and eight on one SM slow each other down)
+    long long walkers = 0;
+    for (long long id : s->running) walkers += s->jobs[id].inst->M.G;
+    const int spread = (int)std::min(8ll, (walkers + s->sms - 1) / s->sms);
     for (size_t i = 0; i < s->running.size(); ++i) {
         Job &j = s->jobs[s->running[i]];
         rewl_s *h = j.inst;
@@ -178,7 +183,7 @@ rewl_status rebuild_tables(rewl_server_s *s) {
         auto &c = s->cls[rewl::sweep_bits(h->M, 32) == 8 ? 1 : 0];
         auto &cw = s->cls[h->M.bits == 8 ? 1 : 0];
         int P = (int)((size_t)s->optin / (size_t)d.lay.stride);
-        P = std::max(1, std::min(P, 8));
+        P = std::max(1, std::min(P, spread));
         for (int g0 = 0; g0 < h->M.G; g0 += P) c.items.push_back({(int)i, g0, std::min(P, h->M.G - g0), 0});
         for (int g = 0; g < h->M.G; ++g) cw.walkers.push_back({(int)i, g});
         c.smem = std::max(c.smem, (size_t)P * (size_t)d.lay.stride);

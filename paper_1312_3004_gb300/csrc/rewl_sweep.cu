@@ -1388,9 +1388,7 @@ Layout make_layout(const Model &M, int S, bool lat_global, int bits) {
 template <int BITS, int S, bool LG>
 cudaError_t launch_lg(const Model &M, const State &St, const SweepPlan &p, cudaStream_t s, bool prepare) {
     const Layout lay = make_layout(M, S, LG, BITS);
-    if (prepare)
-        return cudaFuncSetAttribute(sweep_fast_kernel<BITS, S, LG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)p.smem);
+    if (prepare) return allow_shared((const void *)sweep_fast_kernel<BITS, S, LG>);
     sweep_fast_kernel<BITS, S, LG><<<p.grid, p.threads, p.smem, s>>>(M, St, p.P, lay);
     return cudaGetLastError();
 }
@@ -1429,9 +1427,7 @@ namespace {
 template <int BITS, int S>
 cudaError_t batch_launch_t(const InstDev *inst, const SweepItem *items, int n_items, unsigned int *queue, int grid,
                            int threads, size_t smem, cudaStream_t s, bool prepare) {
-    if (prepare)
-        return cudaFuncSetAttribute(fast::batch_sweep_kernel<BITS, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem);
+    if (prepare) return allow_shared((const void *)fast::batch_sweep_kernel<BITS, S>);
     if (n_items <= 0) return cudaSuccess;
     fast::batch_sweep_kernel<BITS, S><<<grid, threads, smem, s>>>(inst, items, n_items, queue);
     return cudaGetLastError();
@@ -1501,7 +1497,7 @@ bool launch_production_fast(const Model &M, const State &S, int num_sms, size_t 
     if (P < 1) return false;
     const size_t smem = (size_t)P * (size_t)lay.stride;
     auto go = [&](auto kernel) {
-        *err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        *err = allow_shared((const void *)kernel);
         if (*err != cudaSuccess) return;
         kernel<<<(M.G + P - 1) / P, P * 32, smem, s>>>(M, S, P, lay, off_cnt);
         *err = cudaGetLastError();
