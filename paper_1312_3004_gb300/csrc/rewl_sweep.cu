@@ -829,6 +829,7 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
                  (int)(sl0 == nw) - (int)(sd0 == nw) - (int)(su0 == nw);
         // earlier lanes whose flip would change this proposal
         unsigned touch = 0u, twins = d.twins;  // ... ; lanes that propose the same site
+        unsigned t0 = 0u, tr = 0u, tl = 0u, td = 0u, tu = 0u;  // touch, by the site touched
         const uint32_t m0 = lds8(mark_at(site)), mr = lds8(mark_at(nb.r)), ml = lds8(mark_at(nb.l)), md = lds8(mark_at(nb.d)), mu = lds8(mark_at(nb.u));
         if (n < S && j >= n) {  // past the launch's last step: never accepted
             d.blo = (int)0x80000000;
@@ -867,20 +868,28 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             st.pk[j] = (uint32_t)site | ((uint32_t)nw << 20);
             st.pk[S + j] = there;
             __syncwarp(gm);
-            touch = there;
-            if (mr != kNoLane) touch |= st.pk[S + mr];
-            if (ml != kNoLane) touch |= st.pk[S + ml];
-            if (md != kNoLane) touch |= st.pk[S + md];
-            if (mu != kNoLane) touch |= st.pk[S + mu];
-            touch &= lt;
-            if (shared_marks) {  // keep the lanes that do touch
-                unsigned real = 0u;
-                for (unsigned rest = touch; rest; rest &= rest - 1u) {
+            auto at_mark = [&](uint32_t id) {  // (loads without branches)
+                const unsigned x = st.pk[S + (id & (S - 1))] & lt;
+                return id != kNoLane ? x : 0u;
+            };
+            t0 = twins & lt;
+            tr = at_mark(mr);
+            tl = at_mark(ml);
+            td = at_mark(md);
+            tu = at_mark(mu);
+            if (shared_marks) {  // keep the lanes that propose the site itself
+                const unsigned all = tr | tl | td | tu;
+                tr = tl = td = tu = 0u;
+                for (unsigned rest = all; rest; rest &= rest - 1u) {
                     const int ps = (int)(st.pk[__ffs((int)rest) - 1] & 0xfffffu);
-                    if (ps == site || ps == nb.r || ps == nb.l || ps == nb.d || ps == nb.u) real |= rest & (0u - rest);
+                    const unsigned low = rest & (0u - rest);
+                    tr |= ps == nb.r ? low : 0u;
+                    tl |= ps == nb.l ? low : 0u;
+                    td |= ps == nb.d ? low : 0u;
+                    tu |= ps == nb.u ? low : 0u;
                 }
-                touch = real;
             }
+            touch = t0 | tr | tl | td | tu;
             fl = ballot(touch != 0u);
         }
 
@@ -894,26 +903,21 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             moved = 0u;
             if (ballot(need)) {
                 __syncwarp(gm);
-                bool ch = false;
-                if (need) {
-                    int c = cur0, sr = sr0, sl = sl0, sd = sd0, su = su0;
-                    for (unsigned rest = ta; rest; rest &= rest - 1u) {
-                        const uint32_t pk = st.pk[__ffs((int)rest) - 1];
-                        const int ps = (int)(pk & 0xfffffu), pv = (int)(pk >> 20);
-                        c = ps == site ? pv : c;
-                        sr = ps == nb.r ? pv : sr;
-                        sl = ps == nb.l ? pv : sl;
-                        sd = ps == nb.d ? pv : sd;
-                        su = ps == nb.u ? pv : su;
-                    }
-                    last = ta;
-                    cur = c;
-                    const int w = d.v + (d.v >= c);
-                    ch = w != nw;
-                    nw = w;
-                    dE = (int)(sr == c) + (int)(sl == c) + (int)(sd == c) + (int)(su == c) - (int)(sr == w) -
-                         (int)(sl == w) - (int)(sd == w) - (int)(su == w);
-                }
+                // a site's spin: the last accepted flip of it, or as read (for every
+                // lane, without branches: the five chains side by side)
+                auto flip = [&](unsigned t, int was) {
+                    const unsigned a = t & A;
+                    const int x = (int)(st.pk[(31 - __clz((int)a)) & (S - 1)] >> 20);
+                    return a ? x : was;
+                };
+                const int c = flip(t0, cur0), sr = flip(tr, sr0), sl = flip(tl, sl0), sd = flip(td, sd0), su = flip(tu, su0);
+                last = ta;
+                cur = c;
+                const int w = d.v + (d.v >= c);
+                const bool ch = w != nw;
+                nw = w;
+                dE = (int)(sr == c) + (int)(sl == c) + (int)(sd == c) + (int)(su == c) - (int)(sr == w) - (int)(sl == w) -
+                     (int)(sd == w) - (int)(su == w);
                 __syncwarp(gm);
                 if (ch) st.pk[j] = (uint32_t)site | ((uint32_t)nw << 20);
                 moved = ballot(ch);
