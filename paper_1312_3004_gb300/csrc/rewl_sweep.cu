@@ -224,13 +224,16 @@ struct Stage {
 };
 // Entries of the conflict marks: one per site up to kMarks sites.
 constexpr int kMarks = 8192;
+// Lattices in global memory: fewer, so that more walkers fit an SM (q = 10, L = 300,
+// 717 windows of 3: all resident at once, 1.05 -> 0.84 ms a round).
+constexpr int kMarksFar = 2048;
 constexpr uint32_t kNoLane = 255u;
 // ln f from which a lane group counts the batch's own ln f steps in every
 // evaluation (about 60 cycles each) instead of leaving the steps they could
 // decide, about 500 ln f a batch of 32, to the full comparison (about 1000 cycles).
 constexpr double kCountLnf = 0x1p-12;
 constexpr int kCrowded = 300;
-constexpr int kAhead = 4;  // batches drawn at a time
+constexpr int kAhead = 2;  // batches drawn at a time (as fast as 4)
 // Half-units by which D in a batch can miss the true difference beyond the
 // floors of shadow_of: up to 32 adds on either bin, each rounded by at most
 // half a last place (2^8 half-units for values below 2^61 units) and, for an
@@ -1060,20 +1063,24 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         } else {
             const long long F = lds64(at);
             const int c = __popc(steps);
-            if (j < n && (steps & ~le) == 0u) {  // the bin's last step: its lane writes for all of them
-                const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad);
-                long long F2 = (long long)((unsigned long long)F + incF * (unsigned)c);
-                const uint32_t h1 = (uint32_t)((unsigned long long)F >> 32), h2 = (uint32_t)((unsigned long long)F2 >> 32);
-                if (!int_add || (F & 1) || (h2 ^ h1) > h1) {
-                    if (!whole_steps(F, c, LNF, ew, int_add, F2)) {  // binary64 adds
-                        const long long v = exact_steps(F, lgb, b, ew, lnf, c);
-                        F2 = shadow_of(v, ew);
-                        if (F2 & 1) lgb[b] = v;
-                        nseq += (unsigned)c;
-                    }
-                }
+            const bool writer = j < n && (steps & ~le) == 0u;  // the bin's last step: its lane writes for all of them
+            const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad);
+            const long long F2 = (long long)((unsigned long long)F + incF * (unsigned)c);
+            const uint32_t h1 = (uint32_t)((unsigned long long)F >> 32), h2 = (uint32_t)((unsigned long long)F2 >> 32);
+            const bool plain = int_add && !(F & 1) && (h2 ^ h1) <= h1;
+            if (writer) {  // (predicated: no branch)
                 sts64(at, F2);
                 atomicAdd(&hg[b], (uint32_t)c);  // (result not used: the walker does not wait)
+            }
+            if (writer && !plain) {
+                long long F3 = F2;
+                if (!whole_steps(F, c, LNF, ew, int_add, F3)) {  // binary64 adds
+                    const long long v = exact_steps(F, lgb, b, ew, lnf, c);
+                    F3 = shadow_of(v, ew);
+                    if (F3 & 1) lgb[b] = v;
+                    nseq += (unsigned)c;
+                }
+                sts64(at, F3);
             }
         }
         pcur = __shfl_sync(gm, at, n - 1, S);
@@ -1369,7 +1376,7 @@ Layout make_layout(const Model &M, int S, bool lat_global, int bits) {
         l.off_lat = off;
         off += al((M.N * bits + 31) / 32 * 4);
     }
-    l.marks = M.N <= kMarks ? al(M.N) : kMarks;
+    l.marks = M.N <= kMarks ? al(M.N) : lat_global ? kMarksFar : kMarks;
     if (off > kByteStageMax) l.marks = 512;
     // (at least the bytes per walker that decide which windows fit, so that the
     // set of accepted configurations does not depend on the scratch below)
