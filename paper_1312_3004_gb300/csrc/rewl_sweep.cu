@@ -341,18 +341,25 @@ __device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, i
 }
 
 // One lane per walker, its state in global memory: the steps one after another,
-// each proposal drawn (and its spins read) while the previous step waits for its
-// ln g shadow; a spin that the previous step flipped is replaced in registers.
+// the next proposal drawn (and its spins read) while the present step waits for
+// its ln g shadow; a flip of the present step is put into the words read.
 //
-// What bounds it: the instructions of a step and how few warps there are to
-// overlap their latencies (about 12 per SM on 2048 instances).  Hence leading-word
-// decisions, brackets in 32-bit integers, round keys kept in registers, plain
-// stores to the lattice (the thread owns it) and the current bin's shadow and
-// visits in registers until the walker leaves the bin.  The passes over all bins
-// before and after the steps are taken by the warp together, one walker after
-// another, so that the lanes' loads lie side by side (3.1 -> 1.0 ms on 2048
-// instances).  Every thread of a warp calls, live or not.  2048 instances, 56,784
-// walkers, 10^4 steps: 16.1 -> 9.7 ms a round.
+// What bounds it: a step's chain of latencies (a read that misses L1 in some lane,
+// the random words, the decision: 1100 cycles with a warp per scheduler) and, with
+// three warps per scheduler, its 250 instructions (issue 47 % busy).  Hence
+// leading-word decisions, brackets in 32-bit integers, round keys kept in
+// registers, the proposal held as the five words of its spins (a plain store to
+// the lattice, which the thread owns, and one change per word for a flip, taken
+// over only when the proposal is looked at: nothing waits for the reads in the
+// step that issues them) and the current bin's shadow and visits in registers
+// until the walker leaves the bin.  The passes over all bins before and after the
+// steps are taken by the warp together, one walker after another, so that the
+// lanes' loads lie side by side (3.1 -> 1.0 ms on 2048 instances).  Every thread
+// of a warp calls, live or not.  10^4 steps: 2048 instances (56,784 walkers)
+// 16.1 -> 8.7 ms a round, 700 instances 7.9 -> 5.5 ms with words instead of spins.
+// Lattices in shared memory (a word of each lane side by side) were slower, 10.2
+// and 6.9 ms: less L1 for the shadows and fewer warps; so were reads two
+// steps ahead and both possible shadow reads of the next step issued early.
 struct Slow1 {  // what the rare parts of a step need
     long long *lgb;
     double lnf;
@@ -467,10 +474,13 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
     for (int r = 0; r < 20; ++r) asm("" : "+r"(rk[r]));  // kept, not added up again in every block
 
     struct Prop {
-        int site, v, cur, sr, sl, sd, su, T, blo;
-        uint32_t bw;
+        int site, v, T, blo;
+        uint32_t bw, here, wr, wl, wd, wu;  // the words that hold the site and its neighbours
         Site4 nb;
     };
+    constexpr int wsh = BITS == 4 ? 3 : 2;
+    auto same = [](int a, int b) { return (a >> wsh) == (b >> wsh); };
+    auto field = [](uint32_t w, int s) { return (int)(__funnelshift_r(w, 0u, (uint32_t)s * BITS) & ((1u << BITS) - 1u)); };
     auto random = [&](unsigned long long t) {
         return philox((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)g, DOM_WL, rk);
     };
@@ -479,11 +489,11 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         p.site = (int)__umulhi(r.x, (uint32_t)N);
         p.v = (int)__umulhi(r.y, qm1);
         p.nb = nbrs(p.site, L, N, divL);
-        p.cur = spin_get<BITS>(lat, p.site);
-        p.sr = spin_get<BITS>(lat, p.nb.r);
-        p.sl = spin_get<BITS>(lat, p.nb.l);
-        p.sd = spin_get<BITS>(lat, p.nb.d);
-        p.su = spin_get<BITS>(lat, p.nb.u);
+        p.here = lat[p.site >> wsh];
+        p.wr = lat[p.nb.r >> wsh];
+        p.wl = lat[p.nb.l >> wsh];
+        p.wd = lat[p.nb.d >> wsh];
+        p.wu = lat[p.nb.u >> wsh];
         p.T = minus_ln(r.z, r.w);
         lead_bracket(p.T, small_k, tsh, 0, p.blo, p.bw);
     };
@@ -496,22 +506,28 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
     unsigned int nacc = 0;
     unsigned long long t = t_io;
     const unsigned long long t_end = t_io + (unsigned long long)M.K;
-    // Two proposals wait with their spins read, so that a step's reads have two
-    // steps to arrive; both take over a flip in registers.
-    auto flipped = [](Prop &p, int site, int to) {
-        if (p.site == site) p.cur = to;
-        if (p.nb.r == site) p.sr = to;
-        if (p.nb.l == site) p.sl = to;
-        if (p.nb.d == site) p.sd = to;
-        if (p.nb.u == site) p.su = to;
+    // The next proposal is drawn and its words read while a step waits for its
+    // ln g shadow; it takes over the step's flip when it is looked at.
+    auto flipped = [&](Prop &p, int site, uint32_t x) {
+        p.here ^= same(p.site, site) ? x : 0u;
+        p.wr ^= same(p.nb.r, site) ? x : 0u;
+        p.wl ^= same(p.nb.l, site) ? x : 0u;
+        p.wd ^= same(p.nb.d, site) ? x : 0u;
+        p.wu ^= same(p.nb.u, site) ? x : 0u;
     };
-    auto step = [&](const Prop &cp, Prop &n1, Prop &n2) {
-        const int nw = cp.v + (cp.v >= cp.cur);
-        const int dE = (int)(cp.sr == cp.cur) + (int)(cp.sl == cp.cur) + (int)(cp.sd == cp.cur) + (int)(cp.su == cp.cur) -
-                       (int)(cp.sr == nw) - (int)(cp.sl == nw) - (int)(cp.sd == nw) - (int)(cp.su == nw);
+    int fsite = -64;  // the last step's flip (-64: none) and its change of the word
+    uint32_t fx = 0;
+    auto step = [&](Prop &cp, Prop &n1) {
+        flipped(cp, fsite, fx);
+        const int curs = field(cp.here, cp.site);
+        const int sr = field(cp.wr, cp.nb.r), sl = field(cp.wl, cp.nb.l);
+        const int sd = field(cp.wd, cp.nb.d), su = field(cp.wu, cp.nb.u);
+        const int nw = cp.v + (cp.v >= curs);
+        const int dE = (int)(sr == curs) + (int)(sl == curs) + (int)(sd == curs) + (int)(su == curs) -
+                       (int)(sr == nw) - (int)(sl == nw) - (int)(sd == nw) - (int)(su == nw);
         const int En = Eo + dE;
         const long long there = lgf[REWL_IDX(En, -kPad, M.B + kPad, tally.bad)];  // beyond the window: kOutside
-        draw(t + 2ull, n2);  // (past the last step: drawn, never taken)
+        draw(t + 1ull, n1);  // (past the last step: drawn, never taken)
         const long long BF = dE == 0 ? AF : there;
         const int D = (int)(BF >> 32) - (int)(AF >> 32);
         bool acc = D < cp.blo;
@@ -534,19 +550,19 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
             if (!int_add || (cur & 1) || (sh > 0 && ((AF >> 1) & ((1LL << sh) - 1)) != 0))
                 AF = add_1(rare, cur, REWL_IDX(Eb, 0, M.B, tally.bad), AF, int_add);
         }
+        fsite = -64;
         if (acc) {
-            if (BITS == 8) reinterpret_cast<uint8_t *>(lat)[cp.site] = (uint8_t)nw;
-            else atomicXor(&lat[cp.site / per], (uint32_t)(cp.cur ^ nw) << ((cp.site & (per - 1)) * BITS));
+            const uint32_t x = __funnelshift_l(0u, (uint32_t)(curs ^ nw), (uint32_t)cp.site * BITS);
+            lat[cp.site >> wsh] = cp.here ^ x;
             ++nacc;
-            flipped(n1, cp.site, nw);
-            flipped(n2, cp.site, nw);
+            fsite = cp.site;
+            fx = x;
         }
         return ++t == t_end;
     };
-    Prop a, b, c;
+    Prop a, b;
     draw(t, a);
-    draw(t + 1ull, b);
-    while (!step(a, b, c) && !step(b, c, a) && !step(c, a, b)) {
+    while (!step(a, b) && !step(b, a)) {
     }
     lgf[Eo] = AF;
     atomicAdd(&hg[Eo], visits);

@@ -72,3 +72,16 @@ def test_range_of_ln_g(scale, offset, lnf):
 @pytest.mark.parametrize("q,bits", [(10, 4), (10, 8), (30, 8)])
 def test_lattice_placement(lat, q, bits):
     same((q, 15, 4, 0.75, 3, 1e-6, 0.8, 2500, 17), bits, 4, 32, options=[(_lib.OPT_LATTICE, lat)])
+
+
+@pytest.mark.parametrize("lattice", [1, 2])  # in global memory, in shared memory
+@pytest.mark.parametrize("L", [3, 4, 5, 7, 8, 9, 16, 33])  # neighbours in the word of the site, across its edge, the same word twice
+@pytest.mark.parametrize("q,bits", [(2, 8), (10, 4), (20, 8), (2, 4)])
+def test_thread_per_walker_words(L, q, bits, lattice):
+    h = 1 if L < 5 else 3
+    same((q, L, h, 0.75, 2, 1e-6, 0.8, 501, 13), bits, 4, 1, options=[(_lib.OPT_LATTICE, lattice)])
+
+
+@pytest.mark.parametrize("K", [1, 2, 3])
+def test_thread_per_walker_short_rounds(K):
+    same((10, 6, 2, 0.75, 3, 1e-6, 0.8, K, 17), 4, 40, 1)
