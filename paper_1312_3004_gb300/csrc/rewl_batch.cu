@@ -1,8 +1,9 @@
 // rewl_batch.cu -- many independent REWL instances of uneven size (q, L, h, m)
-// in one device allocation, advanced together: one persistent sweep launch per
-// (spin bits, lanes) class takes walker groups of every instance from a device
-// queue, one batched check launch covers every window of every instance, one
-// batched exchange launch every instance; a CUDA graph replays these rounds.
+// in one device allocation, advanced together: persistent sweep launches, one per
+// class of packing and size of walker and side by side, take walker groups of
+// every instance from device queues, one batched check launch covers every window
+// of every instance, one batched exchange launch every instance; a CUDA graph
+// replays these rounds.
 // Every instance computes exactly what it computes alone (its own Philox key,
 // its own state; the kernels run the same block code as the single-instance
 // launches).
@@ -25,8 +26,8 @@ constexpr int kBatchGraphRounds = 4;
 constexpr int kSideStreams = 7;
 // Walkers of a sweep CTA in lane groups: a quarter of what fits its shared memory
 // (and the most a CTA can hold).  A CTA ends with its slowest walker, and small
-// CTAs fill an SM's shared memory: 64 instances (1775 walkers) 1.42 -> @B64@ ms a
-// round, 512 instances 6.9 -> @B512@ ms.
+// CTAs fill an SM's shared memory: 64 instances (1775 walkers) 1.42 -> 1.36 ms a
+// round, 512 instances 6.9 -> 5.7 ms.
 constexpr int kCtaShare = 4;
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -355,7 +356,9 @@ rewl_status rewl_batch_create_ext(const rewl_params *jobs, int n, int spin_bits,
     b->bits_free = spin_bits == 0 && small_q;
     Config c;
     c.lanes = lanes != 0 ? lanes : (walkers >= kWalkerModeMin ? 1 : 32);
-    // a thread per walker reads whole bytes faster than 4-bit fields
+    // (a thread per walker: 8 bits, the packing that saved states of such batches
+    // hold; 4 bits are faster, 8.7 against 9.4 ms a round of 2048 instances, and
+    // rewl_batch_autotune takes them)
     c.bits = spin_bits != 0 ? spin_bits : ((c.lanes == 1 || !small_q) ? 8 : 4);
     size_t off = 0;
     std::vector<size_t> inst_off((size_t)n);

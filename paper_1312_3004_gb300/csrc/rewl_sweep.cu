@@ -604,20 +604,21 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
 // per batch of 32 is 1.0 .. 1.7 at a late ln f and 2 .. 7 at ln f = 1,
 // confirming evaluation included.
 //
-// What bounds it: the latency of one dependent chain per walker (with 7 walkers
-// per SM a batch takes 1740 cycles against 1600 with one walker on the SM alone,
-// and the pipes are a third busy), so every part is chosen for its latency.
-// Measured on GB300, in cycles with their use: popcount 24 (four of them 56),
-// ballot 17 (four 33), match 41 and 11 more per distinct value, shared load 34,
-// store-then-load 42, atomic-then-load 99, leading-zero count 27, a branch on a
-// vote about 45.  Hence ballots and plain stores instead of shared atomics, one
-// branch per evaluation, and the random numbers of four batches at a time (600 ->
-// 290 cycles a batch).  Cycles per batch of 32 at ln f = 2^-20: draws 290,
-// proposals 410, 1.5 evaluations 400, commit 550; at ln f = 1: 4.9 evaluations
-// 1560.  q = 10, L = 80, 1024 walkers, 10^4 steps each, sweep alone: 1.10 -> 0.58 ms
-// in the first rounds (ln f = 1) and 1.03 -> 0.40 ms at ln f = 2^-20, against the
-// step trees that were here before (the decisions of the next five steps at a
-// time, 275 cycles a step).
+// What bounds it: the latency of one dependent chain per walker, so every part is
+// chosen for its latency; with 7 walkers per SM the instructions count as well
+// (60 more in an evaluation cost 20 %).  At ln f = 1 a batch of 32 takes 580 warp
+// instructions (18 a step), the SM issues in 35 % of its cycles, and of the
+// cycles between two instructions of a warp 1.5 are fixed latencies, 1.3 shared
+// memory and the vote units.  Measured on GB300, in cycles with their use:
+// popcount 24 (four of them 56), ballot 17 (four 33), match 41 and 11 more per
+// distinct value, shared load 34, store-then-load 42, atomic-then-load 99,
+// leading-zero count 27, a branch on a vote about 45.  Hence ballots and plain
+// stores instead of shared atomics, one branch per evaluation, flips without
+// branches, and the random numbers of two batches at a time (four: no faster, and
+// more shared memory).  q = 10, L = 80, 1024 walkers, 10^4 steps each, the
+// sweep alone: 1.10 -> 0.57 ms in the first rounds (ln f = 1) and 1.03 -> 0.39 ms
+// at ln f = 2^-20, against the step trees that were here before (the decisions of
+// the next five steps at a time, 275 cycles a step).
 //
 //  * The bin before step j: the batch's start plus the accepted energy changes
 //    of the lanes before it; from four ballots (the bit planes of the changes,
@@ -645,7 +646,7 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
 // not decide.  After every step H(E, O) counts the bin and the class of the
 // majority count O = max_v #{i : s_i = v}: for each value v, two ballots give
 // the steps that gain and lose a spin of it, popcounts its number after each
-// step.  Same workload, 64 classes: 8.4 -> 0.7 ms a round (1024 walkers, reads included) against one thread per
+// step.  Same workload, 64 classes: 8.4 -> 0.65 ms a round (1024 walkers, reads included) against one thread per
 // walker (1690 cycles a step: the binary64 decision and the counts on one chain).
 template <int BITS, int S, bool PROD = false>
 __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb,
