@@ -18,8 +18,9 @@
 //    (about 1e-5 of the decisions) takes the binary64 path exp(a - b) -- the
 //    operation the reference does.
 //  * ln g(E) += ln f is an integer add on the shadow (ln f = 2^-k is a whole
-//    number of half-units); a value that enters the next binade, whose shadow
-//    dropped bits, or an ln f that is no whole number takes binary64 adds.
+//    number of half-units; another ln f adds the same whole number of last places
+//    inside a binade, see whole_steps); a value whose shadow dropped bits and
+//    steps that integers do not give exactly take binary64 adds.
 //  * The S proposals of a batch are resolved together, by fixed-point
 //    iteration over the whole batch (walker_sweep below).
 //  * S = 1: a thread per walker, one step after another (walker_sweep_1).
@@ -92,8 +93,8 @@ __device__ __forceinline__ unsigned long long u53(uint32_t hi, uint32_t lo) {
 constexpr long long kNoReject = 1LL << 62;
 // Shadow value of the bins beyond each end of a window: every proposal there
 // has D >= 2^62 >= t_hi and is rejected like an out-of-window move.  The
-// padding also covers the loads of speculative paths (up to six moves of up
-// to four bins each, see the step tree below).
+// padding also covers the bins that a wrong guess inside a batch can reach
+// (walker_sweep holds them within it).
 constexpr long long kOutside = 0x7fffffffffffffffLL;
 constexpr int kPad = kShadowPad;
 constexpr long long kMant = (1LL << 52) - 1, kHidden = 1LL << 52;
@@ -356,7 +357,7 @@ __device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, i
 // steps are taken by the warp together, one walker after another, so that the
 // lanes' loads lie side by side (3.1 -> 1.0 ms on 2048 instances).  Every thread
 // of a warp calls, live or not.  10^4 steps: 2048 instances (56,784 walkers)
-// 16.1 -> 8.7 ms a round, 700 instances 7.9 -> 5.5 ms with words instead of spins.
+// 16.1 -> 8.7 ms a round, 700 instances 7.9 -> 5.7 ms with words instead of spins.
 // Lattices in shared memory (a word of each lane side by side) were slower, 10.2
 // and 6.9 ms: less L1 for the shadows and fewer warps; so were reads two
 // steps ahead and both possible shadow reads of the next step issued early.
@@ -400,7 +401,6 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
                                uint32_t *__restrict__ hg, int g, int lo, double lnf, int &E_io,
                                unsigned long long &t_io, Tally &tally, bool live) {
     const int N = M.N, L = M.L;
-    constexpr int per = 32 / BITS;
     const uint32_t qm1 = (uint32_t)(M.q - 1), divL = M.divL;
     const long long LNF = __double_as_longlong(lnf);
     if (GLOBAL) {
