@@ -357,7 +357,7 @@ rewl_status rewl_batch_create_ext(const rewl_params *jobs, int n, int spin_bits,
     Config c;
     c.lanes = lanes != 0 ? lanes : (walkers >= kWalkerModeMin ? 1 : 32);
     // (a thread per walker: 8 bits, the packing that saved states of such batches
-    // hold; 4 bits are faster, 8.7 against 9.4 ms a round of 2048 instances, and
+    // hold; 4 bits are faster, 8.4 against 9.1 ms a round of 2048 instances, and
     // rewl_batch_autotune takes them)
     c.bits = spin_bits != 0 ? spin_bits : ((c.lanes == 1 || !small_q) ? 8 : 4);
     size_t off = 0;

@@ -347,7 +347,7 @@ __device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, i
 //
 // What bounds it: a step's chain of latencies (a read that misses L1 in some lane,
 // the random words, the decision: 1100 cycles with a warp per scheduler) and, with
-// three warps per scheduler, its 250 instructions (issue 47 % busy).  Hence
+// three warps per scheduler, its 280 instructions (issue 44 % busy).  Hence
 // leading-word decisions, brackets in 32-bit integers, round keys kept in
 // registers, the proposal held as the five words of its spins (a plain store to
 // the lattice, which the thread owns, and one change per word for a flip, taken
@@ -357,7 +357,8 @@ __device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, i
 // steps are taken by the warp together, one walker after another, so that the
 // lanes' loads lie side by side (3.1 -> 1.0 ms on 2048 instances).  Every thread
 // of a warp calls, live or not.  10^4 steps: 2048 instances (56,784 walkers)
-// 16.1 -> 8.7 ms a round, 700 instances 7.9 -> 5.7 ms with words instead of spins.
+// 16.1 -> 8.4 ms a round (8-bit spins 9.1), 700 instances 7.9 -> 5.5 ms with words
+// instead of spins.
 // Lattices in shared memory (a word of each lane side by side) were slower, 10.2
 // and 6.9 ms: less L1 for the shadows and fewer warps; so were reads two
 // steps ahead and both possible shadow reads of the next step issued early.
@@ -478,22 +479,27 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         uint32_t bw, here, wr, wl, wd, wu;  // the words that hold the site and its neighbours
         Site4 nb;
     };
-    constexpr int wsh = BITS == 4 ? 3 : 2;
-    auto same = [](int a, int b) { return (a >> wsh) == (b >> wsh); };
-    auto field = [](uint32_t w, int s) { return (int)(__funnelshift_r(w, 0u, (uint32_t)s * BITS) & ((1u << BITS) - 1u)); };
+    // sites as bit offsets in the lattice: word s >> 5, bit s (mod 32, as a funnel shift takes it)
+    auto same = [](int a, int b) { return (a >> 5) == (b >> 5); };
+    auto field = [](uint32_t w, int s) { return (int)(__funnelshift_r(w, 0u, (uint32_t)s) & ((1u << BITS) - 1u)); };
+    const int row = L * BITS, all = N * BITS;
     auto random = [&](unsigned long long t) {
         return philox((uint32_t)t, (uint32_t)(t >> 32), (uint32_t)g, DOM_WL, rk);
     };
     auto draw = [&](unsigned long long t, Prop &p) {
         const uint4 r = random(t);
-        p.site = (int)__umulhi(r.x, (uint32_t)N);
+        const int s = (int)__umulhi(r.x, (uint32_t)N), y = (int)__umulhi((uint32_t)s, divL), x = s - y * L;
+        p.site = s * BITS;
         p.v = (int)__umulhi(r.y, qm1);
-        p.nb = nbrs(p.site, L, N, divL);
-        p.here = lat[p.site >> wsh];
-        p.wr = lat[p.nb.r >> wsh];
-        p.wl = lat[p.nb.l >> wsh];
-        p.wd = lat[p.nb.d >> wsh];
-        p.wu = lat[p.nb.u >> wsh];
+        p.nb.r = p.site + (x == L - 1 ? BITS - row : BITS);  // (nbrs)
+        p.nb.l = p.site + (x == 0 ? row - BITS : -BITS);
+        p.nb.d = p.site + (y == L - 1 ? row - all : row);
+        p.nb.u = p.site + (y == 0 ? all - row : -row);
+        p.here = lat[p.site >> 5];
+        p.wr = lat[p.nb.r >> 5];
+        p.wl = lat[p.nb.l >> 5];
+        p.wd = lat[p.nb.d >> 5];
+        p.wu = lat[p.nb.u >> 5];
         p.T = minus_ln(r.z, r.w);
         lead_bracket(p.T, small_k, tsh, 0, p.blo, p.bw);
     };
@@ -515,7 +521,7 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         p.wd ^= same(p.nb.d, site) ? x : 0u;
         p.wu ^= same(p.nb.u, site) ? x : 0u;
     };
-    int fsite = -64;  // the last step's flip (-64: none) and its change of the word
+    int fsite = 0;  // the last step's flip: its site, and its change of the word (0: none)
     uint32_t fx = 0;
     auto step = [&](Prop &cp, Prop &n1) {
         flipped(cp, fsite, fx);
@@ -526,9 +532,9 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
         const int dE = (int)(sr == curs) + (int)(sl == curs) + (int)(sd == curs) + (int)(su == curs) -
                        (int)(sr == nw) - (int)(sl == nw) - (int)(sd == nw) - (int)(su == nw);
         const int En = Eo + dE;
-        const long long there = lgf[REWL_IDX(En, -kPad, M.B + kPad, tally.bad)];  // beyond the window: kOutside
+        long long BF = AF;  // (a proposal that keeps the energy reads nothing)
+        if (dE != 0) BF = lgf[REWL_IDX(En, -kPad, M.B + kPad, tally.bad)];  // beyond the window: kOutside
         draw(t + 1ull, n1);  // (past the last step: drawn, never taken)
-        const long long BF = dE == 0 ? AF : there;
         const int D = (int)(BF >> 32) - (int)(AF >> 32);
         bool acc = D < cp.blo;
         if ((uint32_t)(D - cp.blo) < cp.bw)  // the leading words do not decide
@@ -550,14 +556,10 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
             if (!int_add || (cur & 1) || (sh > 0 && ((AF >> 1) & ((1LL << sh) - 1)) != 0))
                 AF = add_1(rare, cur, REWL_IDX(Eb, 0, M.B, tally.bad), AF, int_add);
         }
-        fsite = -64;
-        if (acc) {
-            const uint32_t x = __funnelshift_l(0u, (uint32_t)(curs ^ nw), (uint32_t)cp.site * BITS);
-            lat[cp.site >> wsh] = cp.here ^ x;
-            ++nacc;
-            fsite = cp.site;
-            fx = x;
-        }
+        fsite = cp.site;
+        fx = acc ? __funnelshift_l(0u, (uint32_t)(curs ^ nw), (uint32_t)cp.site) : 0u;
+        if (acc) lat[cp.site >> 5] = cp.here ^ fx;
+        nacc += acc;
         return ++t == t_end;
     };
     Prop a, b;
