@@ -113,6 +113,13 @@ __device__ __forceinline__ void record_tie(Ctl *ctl, unsigned long long *tlog, u
     }
 }
 
+// Entry of a window's H(E, O) for bin b and class cls.  64 bits: the largest
+// windows have more than 2^31 entries (q = 10, L = 200, one window in 36,001
+// classes: 2.9e9).
+__host__ __device__ constexpr long long heo_index(int b, int n_obins, int cls) {
+    return (long long)b * n_obins + cls;
+}
+
 enum : int { SWEEP_REFERENCE = 0, SWEEP_FAST = 1 };
 
 // Shared-memory layout of one walker in the fast sweep.  The binary64 ln g and

@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(256) production_kernel(Model M, State S, int p
     const long long span = (long long)(M.N - qlo + 1);
     int nmax = 0;
     for (int v = 0; v < M.q; ++v) nmax = max(nmax, cnt[v]);
-    int key = -1;                     // (bin, class) of the current run of steps
+    long long key = -1;               // (bin, class) of the current run of steps
     unsigned long long run = 0, n_acc = 0;
     unsigned int bad = 0;  // failed bounds checks (debug build)
     const uint32_t N = (uint32_t)M.N, qm1 = (uint32_t)(M.q - 1);
@@ -387,7 +387,8 @@ __global__ void __launch_bounds__(256) production_kernel(Model M, State S, int p
                 }
             }
         }
-        const int kk = REWL_IDX(E - lo, 0, M.B, bad) * M.n_obins + (int)((long long)(nmax - qlo) * M.n_obins / span);
+        const long long kk = heo_index(REWL_IDX(E - lo, 0, M.B, bad), M.n_obins,
+                                       (int)((long long)(nmax - qlo) * M.n_obins / span));
         if (kk == key) {
             ++run;
         } else {

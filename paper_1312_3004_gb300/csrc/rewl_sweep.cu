@@ -1073,10 +1073,11 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
             const int cls = narrow ? (int)(x * (uint32_t)st.n_obins / span)
                                    : (int)((unsigned long long)x * (unsigned)st.n_obins / span);
             const int b = REWL_IDX((int)(at - pbase) / 8, 0, M.B, tally.bad);
-            const int key = b * st.n_obins + cls;
-            // one add per run of equal keys, by its last step
-            const int after = __shfl_down_sync(gm, key, 1, S);
-            const bool ends = j < n && (j == n - 1 || after != key);
+            const long long key = heo_index(b, st.n_obins, cls);
+            // one add per run of equal keys, by its last step (keys of neighbouring
+            // steps lie within 5 n_obins < 2^23: the low words tell them apart)
+            const int after = __shfl_down_sync(gm, (int)key, 1, S);
+            const bool ends = j < n && (j == n - 1 || after != (int)key);
             const unsigned before = ballot(ends) & lt;
             if (ends) atomicAdd(&st.heo[key], (unsigned long long)(before ? j - 31 + __clz((int)before) : j + 1));
         } else {

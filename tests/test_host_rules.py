@@ -1,0 +1,10 @@
+"""Index arithmetic and dispatch rules of the kernels, evaluated on the host."""
+from host_rules import evaluate
+
+
+def test_production_histogram_entries_beyond_32_bits(tmp_path):
+    """accepted calls have windows of more than 2^31 entries (bin, class)"""
+    cases = [(80000, 36001, 36000),   # q = 10, L = 200, one window
+             (26886, 80340, 80339),   # q = 255, L = 284, 6 windows that do not overlap
+             (1, 7, 3)]
+    assert evaluate(tmp_path, ["heo_index(%d, %d, %d)" % c for c in cases]) == [b * n + c for b, n, c in cases]
