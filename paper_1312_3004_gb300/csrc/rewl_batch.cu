@@ -115,8 +115,8 @@ rewl_status enqueue_batch_round(rewl_batch_s *b, cudaStream_t s) {
             BATCH_CUDA(rewl::launch_batch_walkers(c.bits, b->d_inst, c.d_walkers, (int)c.walkers.size(), c.grid,
                                                   c.threads, to, false));
         else
-            BATCH_CUDA(rewl::launch_batch_sweep(c.bits, c.lanes, b->d_inst, c.d_items, (int)c.items.size(), c.d_queue,
-                                                c.grid, c.threads, c.smem, to, false));
+            BATCH_CUDA(rewl::launch_batch_sweep(c.bits, b->d_inst, c.d_items, (int)c.items.size(), c.d_queue, c.grid,
+                                                c.threads, c.smem, to, false));
     }
     for (int i = 0; i < sides; ++i) {
         BATCH_CUDA(cudaEventRecord(b->joined[i], b->side[i]));
@@ -313,10 +313,9 @@ rewl_status configure(rewl_batch_s *b, const Config &c) {
         e = cudaMemcpyAsync(sc.d_items, sc.items.data(), sc.items.size() * sizeof(rewl::SweepItem),
                             cudaMemcpyHostToDevice, b->stream);
         if (e != cudaSuccess) break;
-        e = rewl::launch_batch_sweep(sc.bits, sc.lanes, nullptr, nullptr, 0, nullptr, 0, sc.threads, sc.smem, nullptr,
-                                     true);
+        e = rewl::launch_batch_sweep(sc.bits, nullptr, nullptr, 0, nullptr, 0, sc.threads, sc.smem, nullptr, true);
         if (e != cudaSuccess) break;
-        const int per_sm = std::max(1, rewl::batch_sweep_ctas_per_sm(sc.bits, sc.lanes, sc.threads, sc.smem));
+        const int per_sm = std::max(1, rewl::batch_sweep_ctas_per_sm(sc.bits, sc.threads, sc.smem));
         sc.grid = std::min((int)sc.items.size(), per_sm * b->sms);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // tab and wins live on this frame

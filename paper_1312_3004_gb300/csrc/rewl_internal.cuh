@@ -204,12 +204,12 @@ cudaError_t launch_batch_walkers(int bits, const InstDev *inst, const WalkerItem
 int batch_walkers_ctas_per_sm(int bits, int threads);
 cudaError_t launch_batch_check(const InstDev *inst, const WinItem *wins, int n_wins, cudaStream_t s);
 cudaError_t launch_batch_exchange(const InstDev *inst, int n_inst, cudaStream_t s);
-// Persistent batched sweep for one (spin bits, lanes) class: CTAs of `threads`
-// threads with `smem` bytes take items from *queue until n_items are done.
-cudaError_t launch_batch_sweep(int bits, int lanes, const InstDev *inst, const SweepItem *items, int n_items,
-                               unsigned int *queue, int grid, int threads, size_t smem, cudaStream_t s,
-                               bool prepare);
-int batch_sweep_ctas_per_sm(int bits, int lanes, int threads, size_t smem);
+// Persistent batched sweep by lane groups of 32, for the walkers of one spin
+// packing: CTAs of `threads` threads with `smem` bytes take items from *queue
+// until n_items are done.
+cudaError_t launch_batch_sweep(int bits, const InstDev *inst, const SweepItem *items, int n_items, unsigned int *queue,
+                               int grid, int threads, size_t smem, cudaStream_t s, bool prepare);
+int batch_sweep_ctas_per_sm(int bits, int threads, size_t smem);
 
 // Record the message returned by rewl_last_error() on this thread (rewl_host.cu).
 void set_error(const char *msg);

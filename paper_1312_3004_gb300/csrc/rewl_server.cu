@@ -232,8 +232,8 @@ rewl_status rebuild_tables(rewl_server_s *s) {
         if (c.items.empty()) continue;
         SRV_CUDA(cudaMemcpyAsync(c.d_items, c.items.data(), c.items.size() * sizeof(rewl::SweepItem),
                                  cudaMemcpyHostToDevice, s->stream));
-        SRV_CUDA(rewl::launch_batch_sweep(c.bits, 32, nullptr, nullptr, 0, nullptr, 0, c.threads, c.smem, nullptr, true));
-        const int per_sm = std::max(1, rewl::batch_sweep_ctas_per_sm(c.bits, 32, c.threads, c.smem));
+        SRV_CUDA(rewl::launch_batch_sweep(c.bits, nullptr, nullptr, 0, nullptr, 0, c.threads, c.smem, nullptr, true));
+        const int per_sm = std::max(1, rewl::batch_sweep_ctas_per_sm(c.bits, c.threads, c.smem));
         c.grid = std::min((int)c.items.size(), per_sm * s->sms);
     }
     SRV_CUDA(cudaStreamSynchronize(s->stream));
@@ -250,8 +250,8 @@ rewl_status enqueue_round(rewl_server_s *s) {
             SRV_CUDA(rewl::launch_batch_walkers(c.bits, s->d_inst, c.d_walkers, (int)c.walkers.size(), c.wgrid,
                                                 kWalkerThreads, s->stream, false));
         else
-            SRV_CUDA(rewl::launch_batch_sweep(c.bits, 32, s->d_inst, c.d_items, (int)c.items.size(), s->d_queues + k,
-                                              c.grid, c.threads, c.smem, s->stream, false));
+            SRV_CUDA(rewl::launch_batch_sweep(c.bits, s->d_inst, c.d_items, (int)c.items.size(), s->d_queues + k, c.grid,
+                                              c.threads, c.smem, s->stream, false));
     }
     SRV_CUDA(rewl::launch_batch_check(s->d_inst, s->d_wins, s->n_wins, s->stream));
     SRV_CUDA(rewl::launch_batch_exchange(s->d_inst, (int)s->running.size(), s->stream));

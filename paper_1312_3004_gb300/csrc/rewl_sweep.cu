@@ -32,23 +32,18 @@
 namespace rewl {
 namespace fast {
 
-// Philox4x32-10 with the round keys of key word w at rk(w, r), r = 0 .. 9.
-template <typename Keys>
-__device__ __forceinline__ uint4 philox_rounds(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, Keys rk) {
+// Philox4x32-10 with prepared round keys (rk[2 r], rk[2 r + 1] in round r; constant
+// operands in lane groups): 20 wide multiplies and 20 three-input logic operations.
+__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const uint32_t (&rk)[20]) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
         const unsigned long long a = 0xD2511F53ull * c0, b = 0xCD9E8D57ull * c2;  // (one wide multiply each)
-        c0 = (uint32_t)(b >> 32) ^ c1 ^ rk(0, r);
-        c2 = (uint32_t)(a >> 32) ^ c3 ^ rk(1, r);
+        c0 = (uint32_t)(b >> 32) ^ c1 ^ rk[2 * r];
+        c2 = (uint32_t)(a >> 32) ^ c3 ^ rk[2 * r + 1];
         c1 = (uint32_t)b;
         c3 = (uint32_t)a;
     }
     return make_uint4(c0, c1, c2, c3);
-}
-// Lane groups: prepared round keys (constant operands: 20 wide multiplies and
-// 20 three-input logic operations a block).
-__device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const uint32_t (&rk)[20]) {
-    return philox_rounds(c0, c1, c2, c3, [&](int w, int r) { return rk[2 * r + w]; });
 }
 // C blocks of one key, counter words t[c] (low, high) and c2, interleaved so that
 // the rounds of one hide the latency of another.
@@ -1327,8 +1322,8 @@ __global__ void __launch_bounds__(256) production_fast_kernel(Model M, State Sg,
     }
 }
 
-// Persistent batched sweep: each CTA takes the next item from *queue.
-template <int BITS, int S>
+// Persistent batched sweep by lane groups of 32: each CTA takes the next item from *queue.
+template <int BITS>
 __global__ void __launch_bounds__(256) batch_sweep_kernel(const InstDev *inst, const SweepItem *items, int n_items,
                                                           unsigned int *queue) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1342,7 +1337,7 @@ __global__ void __launch_bounds__(256) batch_sweep_kernel(const InstDev *inst, c
         const Model M = inst[it.inst].M;
         const State Sg = inst[it.inst].S;
         const Layout lay = inst[it.inst].lay;
-        sweep_block<BITS, S, false>(M, Sg, it.g0, it.P, lay, smem);
+        sweep_block<BITS, 32, false>(M, Sg, it.g0, it.P, lay, smem);
         __syncthreads();
     }
 }
@@ -1455,62 +1450,23 @@ Layout fast_layout(const Model &M, int lanes, bool lat_global) {
 }
 
 namespace {
-template <int BITS, int S>
-cudaError_t batch_launch_t(const InstDev *inst, const SweepItem *items, int n_items, unsigned int *queue, int grid,
-                           int threads, size_t smem, cudaStream_t s, bool prepare) {
-    if (prepare) return allow_shared((const void *)fast::batch_sweep_kernel<BITS, S>);
-    if (n_items <= 0) return cudaSuccess;
-    fast::batch_sweep_kernel<BITS, S><<<grid, threads, smem, s>>>(inst, items, n_items, queue);
-    return cudaGetLastError();
-}
-template <int BITS>
-cudaError_t batch_dispatch(int lanes, const InstDev *inst, const SweepItem *items, int n_items, unsigned int *queue,
-                           int grid, int threads, size_t smem, cudaStream_t s, bool prepare) {
-    switch (lanes) {
-    case 1: return batch_launch_t<BITS, 1>(inst, items, n_items, queue, grid, threads, smem, s, prepare);
-    case 2: return batch_launch_t<BITS, 2>(inst, items, n_items, queue, grid, threads, smem, s, prepare);
-    case 4: return batch_launch_t<BITS, 4>(inst, items, n_items, queue, grid, threads, smem, s, prepare);
-    case 8: return batch_launch_t<BITS, 8>(inst, items, n_items, queue, grid, threads, smem, s, prepare);
-    case 16: return batch_launch_t<BITS, 16>(inst, items, n_items, queue, grid, threads, smem, s, prepare);
-    default: return batch_launch_t<BITS, 32>(inst, items, n_items, queue, grid, threads, smem, s, prepare);
-    }
-}
-template <int BITS, int S>
-int occupancy_t(int threads, size_t smem) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fast::batch_sweep_kernel<BITS, S>, threads, smem) !=
-        cudaSuccess)
-        return 0;
-    return n;
+const void *batch_sweep(int bits) {
+    return bits == 8 ? (const void *)fast::batch_sweep_kernel<8> : (const void *)fast::batch_sweep_kernel<4>;
 }
 }  // namespace
 
-cudaError_t launch_batch_sweep(int bits, int lanes, const InstDev *inst, const SweepItem *items, int n_items,
-                               unsigned int *queue, int grid, int threads, size_t smem, cudaStream_t s,
-                               bool prepare) {
-    return bits == 8 ? batch_dispatch<8>(lanes, inst, items, n_items, queue, grid, threads, smem, s, prepare)
-                     : batch_dispatch<4>(lanes, inst, items, n_items, queue, grid, threads, smem, s, prepare);
+cudaError_t launch_batch_sweep(int bits, const InstDev *inst, const SweepItem *items, int n_items, unsigned int *queue,
+                               int grid, int threads, size_t smem, cudaStream_t s, bool prepare) {
+    if (prepare) return allow_shared(batch_sweep(bits));
+    if (n_items <= 0) return cudaSuccess;
+    if (bits == 8) fast::batch_sweep_kernel<8><<<grid, threads, smem, s>>>(inst, items, n_items, queue);
+    else fast::batch_sweep_kernel<4><<<grid, threads, smem, s>>>(inst, items, n_items, queue);
+    return cudaGetLastError();
 }
 
-int batch_sweep_ctas_per_sm(int bits, int lanes, int threads, size_t smem) {
-    if (bits == 8) {
-        switch (lanes) {
-        case 1: return occupancy_t<8, 1>(threads, smem);
-        case 2: return occupancy_t<8, 2>(threads, smem);
-        case 4: return occupancy_t<8, 4>(threads, smem);
-        case 8: return occupancy_t<8, 8>(threads, smem);
-        case 16: return occupancy_t<8, 16>(threads, smem);
-        default: return occupancy_t<8, 32>(threads, smem);
-        }
-    }
-    switch (lanes) {
-    case 1: return occupancy_t<4, 1>(threads, smem);
-    case 2: return occupancy_t<4, 2>(threads, smem);
-    case 4: return occupancy_t<4, 4>(threads, smem);
-    case 8: return occupancy_t<4, 8>(threads, smem);
-    case 16: return occupancy_t<4, 16>(threads, smem);
-    default: return occupancy_t<4, 32>(threads, smem);
-    }
+int batch_sweep_ctas_per_sm(int bits, int threads, size_t smem) {
+    int n = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_sweep(bits), threads, smem) == cudaSuccess ? n : 0;
 }
 
 // Whether a walker's production state fits a CTA's shared memory; if so, queue
