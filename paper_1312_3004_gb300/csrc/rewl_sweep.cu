@@ -1327,11 +1327,14 @@ template <int BITS>
 __global__ void __launch_bounds__(256) batch_sweep_kernel(const InstDev *inst, const SweepItem *items, int n_items,
                                                           unsigned int *queue) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int next;
+    // The item's number passes through the first walker's shadow padding, which
+    // sweep_block writes only behind its first barrier: walkers may take all the
+    // shared memory that a CTA can have.
+    volatile int *next = reinterpret_cast<volatile int *>(smem);
     for (;;) {
-        if (threadIdx.x == 0) next = (int)atomicAdd(queue, 1u);
+        if (threadIdx.x == 0) *next = (int)atomicAdd(queue, 1u);
         __syncthreads();
-        const int i = __shfl_sync(0xffffffffu, next, 0);
+        const int i = __shfl_sync(0xffffffffu, *next, 0);
         if (i >= n_items) break;
         const SweepItem it = items[i];
         const Model M = inst[it.inst].M;
@@ -1384,7 +1387,7 @@ Layout make_layout(const Model &M, int S, bool lat_global, int bits) {
         l.stride = 0;
         return l;
     }
-    l.off_lgf = off;
+    l.off_lgf = off;  // (first: batch_sweep_kernel passes an item number through its padding)
     off += al((M.B + 2 * kPad) * 8);
     l.off_lat = -1;
     if (!lat_global) {
