@@ -136,6 +136,9 @@ struct rewl_server_s {
     // the faster is kept.
     int lanes = 32;
     long long tuned_walkers = 0;
+    // every resident walker fits a lane group's shared memory; while one does not (a
+    // large lattice beside a wide window) the rounds run a thread per walker
+    bool groups_fit = true;
     unsigned int *d_queues = nullptr;
     int sms = 0, optin = 0;
     // counters
@@ -171,6 +174,7 @@ rewl_status rebuild_tables(rewl_server_s *s) {
     long long walkers = 0;
     for (long long id : s->running) walkers += s->jobs[id].inst->M.G;
     const int spread = (int)std::min(8ll, (walkers + s->sms - 1) / s->sms);
+    s->groups_fit = true;
     for (size_t i = 0; i < s->running.size(); ++i) {
         Job &j = s->jobs[s->running[i]];
         rewl_s *h = j.inst;
@@ -182,10 +186,14 @@ rewl_status rebuild_tables(rewl_server_s *s) {
         for (int w = 0; w < h->M.h; ++w) wins.push_back({(int)i, w});
         auto &c = s->cls[rewl::sweep_bits(h->M, 32) == 8 ? 1 : 0];
         auto &cw = s->cls[h->M.bits == 8 ? 1 : 0];
+        for (int g = 0; g < h->M.G; ++g) cw.walkers.push_back({(int)i, g});
         int P = (int)((size_t)s->optin / (size_t)d.lay.stride);
+        if (P < 1) {
+            s->groups_fit = false;
+            continue;
+        }
         P = std::max(1, std::min(P, spread));
         for (int g0 = 0; g0 < h->M.G; g0 += P) c.items.push_back({(int)i, g0, std::min(P, h->M.G - g0), 0});
-        for (int g = 0; g < h->M.G; ++g) cw.walkers.push_back({(int)i, g});
         c.smem = std::max(c.smem, (size_t)P * (size_t)d.lay.stride);
         c.threads = std::max(c.threads, P * 32);
     }
@@ -381,8 +389,8 @@ rewl_status rewl_server_step(rewl_server_t s, long long rounds, int *n_running, 
             if (st) return st;
             long long walkers = 0;
             for (long long id : s->running) walkers += s->jobs[id].inst->M.G;
-            if (walkers < kTuneMinWalkers) {
-                s->lanes = 32;
+            if (!s->groups_fit || walkers < kTuneMinWalkers) {
+                s->lanes = s->groups_fit ? 32 : 1;
                 s->tuned_walkers = 0;
             } else if (s->tuned_walkers == 0 || 2 * walkers > 3 * s->tuned_walkers ||
                        3 * walkers < 2 * s->tuned_walkers) {

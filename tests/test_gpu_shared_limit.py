@@ -42,3 +42,21 @@ def test_batch():
     a.run(2)
     for f in ("spins", "energy", "steps", "lng", "hist", "mask"):
         assert np.array_equal(b.instance(0).get(f), a.get(f)), f
+
+
+def test_server_job_whose_lattice_does_not_fit_beside_its_window():
+    """a single handle keeps such a lattice in global memory; the server runs
+    its jobs a thread per walker while one of them is resident"""
+    big = dict(q=10, L=200, h=9, overlap=0.75, m=1, lnf_final=1e-6, flatness=0.8, exchange_interval=20, seed=3)
+    small = dict(big, L=8, h=2)
+    s = Server(256 << 20, max_jobs=4)
+    i = s.submit(**small)
+    s.step(1)
+    k = s.submit(**big)
+    s.step(3)
+    assert s.mapping()[0] == 1
+    assert s.poll(k) == "running" and s.job_info(k)["rounds"] == 3 and s.job_info(i)["rounds"] == 4
+    assert s.job_info(k)["flips"] == 3 * 20 * 9
+    s.cancel(k)
+    s.step(1)
+    assert s.mapping()[0] == 32 and s.job_info(i)["rounds"] == 5
