@@ -195,6 +195,10 @@ Layout fast_layout(const Model &M, int lanes, bool lat_global = false);
 int sweep_bits(const Model &M, int lanes, bool lat_global = false);
 // A lattice above this many bytes stays in global memory in the fast sweep.
 constexpr int kSharedLatticeMax = 16384;
+// Whether the sweeps take decisions on the leading 32-bit words of ln g shadows
+// in half-units of 2^-k first: the draws' 2^-26 are shifted right by 58 - k bits,
+// which a 32-bit word allows from 1 to 31.
+__host__ __device__ constexpr bool leading_words(int k) { return k >= 27 && k <= 57; }
 // Sentinel bins beyond each end of a window in the ln g shadow.
 constexpr int kShadowPad = 24;
 // The batched one-lane sweep: every walker's state in global memory, a thread

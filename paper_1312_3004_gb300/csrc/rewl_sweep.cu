@@ -283,11 +283,12 @@ __device__ __forceinline__ int minus_ln(uint32_t hi, uint32_t lo) {
 // decide (the true difference D 2^-32 lies strictly within 1 of the difference of
 // the leading words, kSlack is far below a leading word's unit, and out of the
 // window the difference is at least 2^30 - 2, above every T at tsh = 58 - k >= 1).
-// small_k: the draws' 2^-26 fits that unit, 26 <= k <= 57; loose: more units.
+// small_k: leading_words(k); loose: more units.
 __device__ __forceinline__ void lead_bracket(int T, bool small_k, int tsh, int loose, int &blo, uint32_t &bw) {
     const int mg = (T >> 18) + 260;  // (Lf + 1) 2^-18, rounded up
     blo = ((T - mg) >> tsh) - 1 - loose;
-    bw = (uint32_t)(((T + mg) >> tsh) + 3 + loose - blo);
+    const int up = (int)((uint32_t)T + (uint32_t)mg);  // (kTiny: not used)
+    bw = (uint32_t)((up >> tsh) + 3 + loose - blo);
     if (T == kTiny || !small_k) {
         blo = small_k ? -2 : -0x7fffffff;
         bw = 0xfffffff0u;
@@ -433,7 +434,7 @@ __device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long 
     rare.lnf = lnf;
     rare.ew = max(1, (int)(__double_as_longlong(reach) >> 52) - 7);
     rare.k = 1076 - rare.ew;
-    rare.small_k = rare.k >= 26 && rare.k <= 57;
+    rare.small_k = leading_words(rare.k);
     const bool small_k = rare.small_k;
     const int tsh = small_k ? 58 - rare.k : 0;
     for (unsigned rest = lanes; rest; rest &= rest - 1u) {
@@ -714,8 +715,8 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
     }
     // Decisions are first taken on the leading 32-bit words of the shadows, in
     // units of 2^(32 - k); where those cannot decide, on all 64 bits (see
-    // `bracket` below).  small_k: the draws' 2^-26 fits that unit.
-    const bool small_k = __all_sync(gm, k >= 26 && k <= 57 && !blind);
+    // `bracket` below).
+    const bool small_k = __all_sync(gm, leading_words(k) && !blind);
     const int tsh = small_k ? 58 - k : 0;
     // At a large ln f many evaluations have to count the batch's own ln f steps:
     // they all do, in leading words (loose: with up to 32 units for what those cut off).

@@ -8,3 +8,9 @@ def test_production_histogram_entries_beyond_32_bits(tmp_path):
              (26886, 80340, 80339),   # q = 255, L = 284, 6 windows that do not overlap
              (1, 7, 3)]
     assert evaluate(tmp_path, ["heo_index(%d, %d, %d)" % c for c in cases]) == [b * n + c for b, n, c in cases]
+
+
+def test_leading_words_are_shifted_by_less_than_their_width(tmp_path):
+    ks = range(-200, 300)
+    taken = [k for k, ok in zip(ks, evaluate(tmp_path, ["leading_words(%d)" % k for k in ks])) if ok]
+    assert taken and all(0 < 58 - k < 32 for k in taken)
