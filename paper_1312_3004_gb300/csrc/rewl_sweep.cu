@@ -351,7 +351,8 @@ __device__ __forceinline__ bool whole_steps(long long F, int c, long long LNF, i
 // step that issues them) and the current bin's shadow and visits in registers
 // until the walker leaves the bin.  The passes over all bins before and after the
 // steps are taken by the warp together, one walker after another, so that the
-// lanes' loads lie side by side (3.1 -> 1.0 ms on 2048 instances).  Every thread
+// lanes' loads lie side by side (3.1 -> 1.0 ms on 2048 instances; so a walker's ln g
+// has more than one name, and lgb is not __restrict__).  Every thread
 // of a warp calls, live or not.  10^4 steps: 2048 instances (56,784 walkers)
 // 16.1 -> 8.4 ms a round (8-bit spins 9.1), 700 instances 7.9 -> 5.5 ms with words
 // instead of spins.
@@ -394,7 +395,7 @@ __device__ __noinline__ long long add_1(Slow1 &s, long long F, int b, long long 
 constexpr int kInFlight = 8;  // loads of such a pass in flight per lane
 
 template <int BITS, bool GLOBAL>
-__device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long long *__restrict__ lgb, long long *lgf,
+__device__ void walker_sweep_1(const Model &M, uint32_t *__restrict__ lat, long long *lgb, long long *lgf,
                                uint32_t *__restrict__ hg, int g, int lo, double lnf, int &E_io,
                                unsigned long long &t_io, Tally &tally, bool live) {
     const int N = M.N, L = M.L;
