@@ -104,24 +104,25 @@ rewl_status enqueue_batch_round(rewl_batch_s *b, cudaStream_t s) {
     // the sweep launches side by side: the first on s, the others on streams that
     // start behind s and that s waits for
     const int sides = std::min((int)b->classes.size() - 1, kSideStreams);
-    if (sides > 0) {
-        BATCH_CUDA(cudaEventRecord(b->forked, s));
-        for (int i = 0; i < sides; ++i) BATCH_CUDA(cudaStreamWaitEvent(b->side[i], b->forked, 0));
-    }
-    for (size_t k = 0; k < b->classes.size(); ++k) {
+    if (sides > 0) BATCH_CUDA(cudaEventRecord(b->forked, s));
+    cudaError_t e = cudaSuccess;  // (of the first call that failed: the streams are joined all the same)
+    auto call = [&](cudaError_t x) { e = e == cudaSuccess ? x : e; };
+    for (int i = 0; i < sides; ++i) call(cudaStreamWaitEvent(b->side[i], b->forked, 0));
+    for (size_t k = 0; k < b->classes.size() && e == cudaSuccess; ++k) {
         SweepClass &c = b->classes[k];
         const cudaStream_t to = k == 0 ? s : b->side[(k - 1) % kSideStreams];
         if (c.lanes == 1)
-            BATCH_CUDA(rewl::launch_batch_walkers(c.bits, b->d_inst, c.d_walkers, (int)c.walkers.size(), c.grid,
-                                                  c.threads, to, false));
+            call(rewl::launch_batch_walkers(c.bits, b->d_inst, c.d_walkers, (int)c.walkers.size(), c.grid, c.threads, to,
+                                            false));
         else
-            BATCH_CUDA(rewl::launch_batch_sweep(c.bits, b->d_inst, c.d_items, (int)c.items.size(), c.d_queue, c.grid,
-                                                c.threads, c.smem, to, false));
+            call(rewl::launch_batch_sweep(c.bits, b->d_inst, c.d_items, (int)c.items.size(), c.d_queue, c.grid, c.threads,
+                                          c.smem, to, false));
     }
     for (int i = 0; i < sides; ++i) {
-        BATCH_CUDA(cudaEventRecord(b->joined[i], b->side[i]));
-        BATCH_CUDA(cudaStreamWaitEvent(s, b->joined[i], 0));
+        call(cudaEventRecord(b->joined[i], b->side[i]));
+        call(cudaStreamWaitEvent(s, b->joined[i], 0));
     }
+    if (e != cudaSuccess) return fail(REWL_ERR_CUDA, "sweep launches: %s", cudaGetErrorString(e));
     BATCH_CUDA(rewl::launch_batch_check(b->d_inst, b->d_wins, b->n_wins, s));
     BATCH_CUDA(rewl::launch_batch_exchange(b->d_inst, (int)b->inst.size(), s));
     return REWL_OK;
