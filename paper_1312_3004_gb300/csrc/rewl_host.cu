@@ -772,11 +772,11 @@ rewl_status rewl_get_field(rewl_t h, int field, void *out, size_t bytes) {
     rewl_status st = field_geometry(h, field, &dev, &need);
     if (st) return st;
     if (bytes != need) return fail(REWL_ERR_ARG, "field %d needs %zu bytes, got %zu", field, need, bytes);
-    rewl::host::touch_pages(out, bytes);
     if (field == REWL_FIELD_SPINS) {
         uint8_t *tmp = nullptr;
         REWL_CUDA(cudaMallocAsync((void **)&tmp, need, h->stream));
         cudaError_t e = rewl::launch_get_spins(h->M, h->S, tmp, h->stream);
+        rewl::host::touch_pages(out, bytes);  // (while the kernel runs)
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, need, cudaMemcpyDeviceToHost, h->stream);
         cudaFreeAsync(tmp, h->stream);
         if (e != cudaSuccess) return fail(REWL_ERR_CUDA, "spins: %s", cudaGetErrorString(e));
@@ -792,6 +792,7 @@ rewl_status rewl_get_field(rewl_t h, int field, void *out, size_t bytes) {
         for (size_t g = 0; g < (size_t)h->M.G; ++g) o[g] = cfgE[slot[g]];
         return REWL_OK;
     } else {
+        rewl::host::touch_pages(out, bytes);
         REWL_CUDA(cudaMemcpyAsync(out, dev, need, cudaMemcpyDeviceToHost, h->stream));
     }
     REWL_CUDA(cudaStreamSynchronize(h->stream));

@@ -14,3 +14,18 @@ def test_leading_words_are_shifted_by_less_than_their_width(tmp_path):
     ks = range(-200, 300)
     taken = [k for k, ok in zip(ks, evaluate(tmp_path, ["leading_words(%d)" % k for k in ks])) if ok]
     assert taken and all(0 < 58 - k < 32 for k in taken)
+
+
+def test_faulting_in_a_result_buffer_keeps_what_it_holds(tmp_path):
+    """a read that fails later leaves the caller's buffer as it was; every page is
+    looked at once, whatever the alignment"""
+    assert evaluate(tmp_path, [r"""([] {
+        std::vector<unsigned char> v(1000003);
+        for (size_t i = 0; i < v.size(); ++i) v[i] = (unsigned char)(i * 7 + 1);
+        rewl::host::fault_in(v.data() + 1, v.size() - 1);
+        rewl::host::fault_in(v.data(), 0);
+        rewl::host::fault_in(v.data() + 5, 1);
+        for (size_t i = 0; i < v.size(); ++i)
+            if (v[i] != (unsigned char)(i * 7 + 1)) return 0;
+        return 1;
+    })()"""]) == [1]
