@@ -180,7 +180,9 @@ cudaError_t launch_exchange(const Model &M, const State &S, cudaStream_t s);
 // with H(E, O) accumulated per window.
 cudaError_t launch_count_spins(const Model &M, const State &S, cudaStream_t s);
 cudaError_t launch_production_sweep(const Model &M, const State &S, cudaStream_t s);
-// (lane groups; false: a walker's state does not fit in shared memory)
+// (lane groups; false: a walker's state does not fit in shared memory, or a thread
+// per walker is faster)
+bool production_lane_groups(const Model &M, int num_sms, int P, int ctas_per_sm);
 bool launch_production_fast(const Model &M, const State &S, int num_sms, size_t smem_optin, cudaStream_t s,
                             cudaError_t *err);
 cudaError_t launch_set_spins(const Model &M, const State &S, const uint8_t *spins_dev, cudaStream_t s);

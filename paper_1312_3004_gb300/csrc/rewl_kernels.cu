@@ -303,8 +303,9 @@ __global__ void __launch_bounds__(256) sweep_kernel(Model M, State S, int P) {
 // counts the current energy and the class of the majority count
 // O = max_v #{i : s_i = v} of the configuration, one of n_obins equal integer
 // classes of [ceil(N/q), N].  Every window runs, finished or not; H stays 0.
-// This form serves windows too wide for shared memory (the other one is the
-// lane groups' PROD sweep in rewl_sweep.cu).
+// This form serves windows too wide for shared memory, and many walkers of many
+// values (production_lane_groups; the other form is the lane groups' PROD sweep,
+// both in rewl_sweep.cu).
 // One thread per walker; lattice, ln g and the spin counts of the walker's
 // configuration buffer in global memory (the thread owns that buffer for the
 // launch); runs of equal (E, O) are added to H(E, O) with one atomic each.
@@ -885,7 +886,8 @@ cudaError_t launch_production_sweep(const Model &M, const State &S, cudaStream_t
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    // a thread per walker only where a window is too wide for shared memory
+    // a thread per walker where a window is too wide for shared memory, and where there
+    // are so many walkers and values that it is the faster form
     if (launch_production_fast(M, S, sms, (size_t)optin, s, &e)) return e;
     int per = (M.G + sms - 1) / sms;  // walkers per CTA: one CTA per SM
     if (per > 256) per = 256;

@@ -24,8 +24,8 @@
 //  * The S proposals of a batch are resolved together, by fixed-point
 //    iteration over the whole batch (walker_sweep below).
 //  * S = 1: a thread per walker, one step after another (walker_sweep_1).
+#include <algorithm>
 #include <cstdint>
-#include <type_traits>
 
 #include "rewl_internal.cuh"
 
@@ -1474,9 +1474,35 @@ int batch_sweep_ctas_per_sm(int bits, int threads, size_t smem) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_sweep(bits), threads, smem) == cudaSuccess ? n : 0;
 }
 
-// Whether a walker's production state fits a CTA's shared memory; if so, queue
-// the sweep (P walkers a CTA, one CTA per SM while the walkers last: their
-// chains, not a pipe, set the rate).
+// Production by lane groups or by a thread per walker: which is faster, from what both
+// took on GB300 (q = 3 .. 255, L = 16 .. 200, 3 to 860 walkers per SM; estimates in
+// microseconds per 1000 steps of every walker, most within 10 %).
+//  * Lane groups go in waves of the CTAs that are resident together.  A wave of r
+//    walkers per SM takes 43 + 1.1 q (each value's count is looked at by every batch:
+//    latency up to about 10 walkers per SM, issue slots above), and 20 to set up.
+//  * A thread per walker takes one chain of steps, 700 for a few walkers per SM; in
+//    full warps the lanes diverge (to 1700 at 40 walkers per SM), more warps share the
+//    SM, and large lattices and many counts leave the caches.
+// q = 10, L = 80: groups up to 340 walkers per SM (7.47 against 9.18 ms a round of 3000
+// steps; at 674 14.3 against 13.2); q = 80: up to 110 (5.8 / 6.6; at 168 8.7 / 7.8);
+// q = 255: up to 27 (4.1 / 4.9; at 54 7.3 / 6.1, at 674 84.8 / 21.2).
+bool production_lane_groups(const Model &M, int num_sms, int P, int ctas_per_sm) {
+    auto wave = [&](double r) {
+        return 43.0 + 20e3 / M.K + std::max(0.0, 0.9 * (r - 8.0)) + M.q * std::max(1.1, 0.112 * r);
+    };
+    const long long ctas = (M.G + P - 1) / P, at_once = (long long)num_sms * ctas_per_sm, rest = ctas % at_once;
+    double groups = (double)(ctas / at_once) * wave((double)P * ctas_per_sm);
+    if (rest) groups += wave((double)P * (double)((rest + num_sms - 1) / num_sms));
+    const double w = (double)M.G / num_sms;
+    const double chain = 700.0 + 25.0 * std::min(w, 40.0) + 3.6 * w;
+    const double counts = 1.0 + 0.0015 * M.q * std::min(std::max(0.0, (w - 30.0) / 120.0), 1.0);
+    const double lattices = 0.85 + M.wpc * 4 / 42000.0;
+    return groups <= chain * counts * lattices;
+}
+
+// If a walker's production state fits a CTA's shared memory and lane groups are the
+// faster form, queue the sweep (P walkers a CTA, one CTA per SM while the walkers
+// last: their chains, not a pipe, set the rate).
 bool launch_production_fast(const Model &M, const State &S, int num_sms, size_t smem_optin, cudaStream_t s,
                             cudaError_t *err) {
     const bool lg = M.wpc * 4 > kSharedLatticeMax;
@@ -1488,15 +1514,22 @@ bool launch_production_fast(const Model &M, const State &S, int num_sms, size_t 
     P = min(min(P, 8), (M.G + num_sms - 1) / num_sms);
     if (P < 1) return false;
     const size_t smem = (size_t)P * (size_t)lay.stride;
+    bool queued = true;
     auto go = [&](auto kernel) {
         *err = allow_shared((const void *)kernel);
         if (*err != cudaSuccess) return;
+        int per_sm = 1;
+        if ((M.G + P - 1) / P > num_sms)
+            *err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, P * 32, smem);
+        if (*err != cudaSuccess) return;
+        queued = production_lane_groups(M, num_sms, P, max(per_sm, 1));
+        if (!queued) return;
         kernel<<<(M.G + P - 1) / P, P * 32, smem, s>>>(M, S, P, lay, off_cnt);
         *err = cudaGetLastError();
     };
     if (lg) bits == 8 ? go(fast::production_fast_kernel<8, true>) : go(fast::production_fast_kernel<4, true>);
     else bits == 8 ? go(fast::production_fast_kernel<8, false>) : go(fast::production_fast_kernel<4, false>);
-    return true;
+    return queued;
 }
 
 cudaError_t launch_batch_walkers(int bits, const InstDev *inst, const WalkerItem *items, int n_items, int grid,

@@ -17,7 +17,7 @@ static const size_t kShared = 232448;
 static Model model(int q, int L, int h, int W, int m, int bits) {
     Model M{};
     M.q = q, M.L = L, M.N = L * L, M.W = W, M.B = W + 1, M.h = h, M.m = m, M.G = h * m;
-    M.bits = bits, M.wpc = (M.N * bits + 31) / 32;
+    M.bits = bits, M.wpc = (M.N * bits + 31) / 32, M.K = 3000;
     return M;
 }
 int main() {

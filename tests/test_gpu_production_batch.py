@@ -81,3 +81,8 @@ def test_ln_g_that_is_no_number(bad):
     gpu.production_run(1)
     assert np.array_equal(gpu.get("energy"), energy) and np.array_equal(gpu.get("spins"), spins)
     assert int(gpu.heo().sum()) == 2 * K
+
+
+@pytest.mark.parametrize("L,h,m", [(10, 8, 64), (12, 40, 256)])  # lane groups; a thread per walker is the faster form
+def test_many_walkers_of_many_values(L, h, m):
+    compare((255, L, h, 0.75, m, 1e-6, 0.8, 40, 7), 8, 13, rounds=2, wl=1)

@@ -29,3 +29,18 @@ def test_faulting_in_a_result_buffer_keeps_what_it_holds(tmp_path):
             if (v[i] != (unsigned char)(i * 7 + 1)) return 0;
         return 1;
     })()"""]) == [1]
+
+
+def test_production_form_is_the_faster_one(tmp_path):
+    """(q, L, h, W, m, walkers a CTA, CTAs per SM): the form that was measured the
+    faster by a fifth or more"""
+    groups = [(10, 80, 64, 766, 16, 7, 1), (10, 80, 64, 766, 256, 8, 1), (10, 300, 717, 1000, 3, 8, 1),
+              (255, 80, 64, 766, 32, 8, 1), (255, 200, 200, 1578, 32, 8, 1), (80, 80, 200, 253, 64, 8, 1),
+              (255, 40, 64, 191, 64, 8, 3), (30, 40, 256, 50, 256, 8, 3), (10, 40, 512, 25, 256, 8, 3),
+              (255, 80, 8, 4655, 128, 4, 1), (10, 16, 100, 20, 256, 8, 3), (80, 80, 2, 10240, 256, 2, 1)]
+    threads = [(255, 80, 64, 766, 256, 8, 1), (255, 80, 8, 4655, 256, 4, 1), (80, 128, 64, 1955, 256, 5, 1),
+               (255, 40, 64, 191, 256, 8, 3), (80, 40, 256, 50, 256, 8, 3), (30, 80, 400, 127, 256, 8, 1),
+               (255, 200, 200, 1578, 128, 8, 1), (255, 16, 100, 20, 256, 8, 3)]
+    rule = ["production_lane_groups(model(%d, %d, %d, %d, %d, %d), kSms, %d, %d)"
+            % (q, L, h, W, m, 4 if q <= 16 else 8, P, c) for q, L, h, W, m, P, c in groups + threads]
+    assert evaluate(tmp_path, rule) == [1] * len(groups) + [0] * len(threads)
