@@ -223,6 +223,13 @@ constexpr int kMarks = 8192;
 // Lattices in global memory: fewer, so that more walkers fit an SM (q = 10, L = 300,
 // 717 windows of 3: all resident at once, 1.05 -> 0.84 ms a round).
 constexpr int kMarksFar = 2048;
+// Narrow lane groups: a CTA holds 256 / S walkers, and their memory is what limits it.
+// Eight lanes take at most 2048 entries (1024 beside lattices in global memory) and
+// leave larger lattices packed, two and four take the bytes that a walker is granted
+// anyway (make_layout).  q = 10, L = 80, 64 windows of 32, 1000 steps, with an entry
+// and a byte per site -> so: 8 lanes 0.90 -> 0.54 ms, 4 lanes 2.34 -> 1.30, 2 lanes 5.5 -> 3.0
+// (windows of 16, where all fit: 0.507 -> 0.523).
+constexpr int kMarksNarrow = 2048;
 constexpr uint32_t kNoLane = 255u;
 // ln f from which a lane group counts the batch's own ln f steps in every
 // evaluation (about 60 cycles each) instead of leaving the steps they could
@@ -964,6 +971,7 @@ __device__ __forceinline__ void walker_sweep(const Model &M, uint32_t *__restric
         // the same for every evaluation at a large ln f: in a fifth of the
         // instructions, by a match (11 cycles per distinct bin) and a table
         auto counted_now = [&]() {
+            if (S == 2) return j == 1 ? (int)(to == pre) - 1 : 0;  // (the second step starts from the first one's bin)
             const unsigned here = __match_any_sync(gm, pre) >> gbase;
             const uint32_t slot = tab_at(pre);
             __syncwarp(gm);
@@ -1369,14 +1377,13 @@ __global__ void __launch_bounds__(256) batch_walker_kernel(const InstDev *inst, 
 
 // Bits per spin of a lattice staged in shared memory: bytes, one load per spin
 // (4-bit fields take a shift and a mask more for each of a proposal's five
-// spins), unless the walker's state is so large that the wider lattice would
-// cost walkers per SM.
+// spins), up to this many bytes for the walker; narrow lane groups: see kMarksNarrow.
 constexpr int kByteStageMax = 96 * 1024;
 
 Layout make_layout(const Model &M, int S, bool lat_global, int bits);
 
 int stage_bits(const Model &M, int S, bool lat_global) {
-    if (M.bits == 8 || lat_global || S == 1) return M.bits;
+    if (M.bits == 8 || lat_global || S <= 4 || (S == 8 && M.N > kMarksNarrow)) return M.bits;
     return make_layout(M, S, false, 8).stride <= kByteStageMax ? 8 : 4;
 }
 
@@ -1396,11 +1403,17 @@ Layout make_layout(const Model &M, int S, bool lat_global, int bits) {
         l.off_lat = off;
         off += al((M.N * bits + 31) / 32 * 4);
     }
-    l.marks = M.N <= kMarks ? al(M.N) : lat_global ? kMarksFar : kMarks;
-    if (off > kByteStageMax) l.marks = 512;
     // (at least the bytes per walker that decide which windows fit, so that the
     // set of accepted configurations does not depend on the scratch below)
-    const int fits = off + (S > 1 ? al((S + 8) * 16) + al((S + 8) * 4) + al(2 * ((min(M.N, 8192) + 31) / 32) * 4) : 0);
+    const int least = S > 1 ? al((S + 8) * 16) + al((S + 8) * 4) + al(2 * ((min(M.N, 8192) + 31) / 32) * 4) : 0;
+    const int fits = off + least;
+    const int queues = al(kAhead * S * 8) + al(2 * S * 4) + al(8 * S * 4);
+    int most = lat_global ? kMarksFar : kMarks;
+    if (S == 8) most = lat_global ? kMarksNarrow / 2 : kMarksNarrow;
+    if (S <= 4)
+        for (most = 512; 2 * most <= least - queues;) most *= 2;
+    l.marks = M.N <= (S > 8 ? kMarks : most) ? al(M.N) : most;
+    if (off > kByteStageMax) l.marks = 512;
     if (S > 1) {
         l.off_ring = off;
         off += al(kAhead * S * 8);

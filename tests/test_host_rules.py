@@ -44,3 +44,19 @@ def test_production_form_is_the_faster_one(tmp_path):
     rule = ["production_lane_groups(model(%d, %d, %d, %d, %d, %d), kSms, %d, %d)"
             % (q, L, h, W, m, 4 if q <= 16 else 8, P, c) for q, L, h, W, m, P, c in groups + threads]
     assert evaluate(tmp_path, rule) == [1] * len(groups) + [0] * len(threads)
+
+
+def test_narrow_lane_groups_hold_the_walkers_that_an_sm_is_given(tmp_path):
+    """walkers per CTA, against what the bytes that decide which windows fit allow"""
+    def granted(L, B, m_per_sm, lanes):
+        al = lambda x: -(-x // 16) * 16
+        n = L * L
+        per = al((B + 48) * 8) + al(n // 2) + al((lanes + 8) * 16) + al((lanes + 8) * 4) + al(2 * (-(-min(n, 8192) // 32)) * 4)
+        return min(232448 // per, 256 // lanes, m_per_sm)
+
+    cases = [(L, h, W, m, lanes) for L, h, W, ms in ((80, 64, 764, (16, 32, 64, 128)), (80, 173, 291, (16, 64)),
+                                                     (40, 41, 291, (64, 200)), (16, 40, 48, (64, 256)))
+             for m in ms for lanes in (2, 4, 8)]
+    P = evaluate(tmp_path, ["plan_sweep(model(10, %d, %d, %d, %d, 4), kSms, kShared, SWEEP_FAST, %d).P" % c for c in cases])
+    for (L, h, W, m, lanes), p in zip(cases, P):
+        assert p >= 0.9 * granted(L, W + 1, -(-h * m // 152), lanes), (L, h, m, lanes, p)
