@@ -517,8 +517,13 @@ __device__ __forceinline__ bool flat_by_walkers(const Model &M, const uint32_t *
     int over = 0;
     for (int b = tid; b < B; b += CHECK_THREADS) {
         uint32_t any = 0;  // (the top bit: a bin at 2^31 visits)
+        int k = 0;
 #pragma unroll 8
-        for (int k = 0; k < m; ++k) any |= H[(size_t)k * B + b];
+        for (; k < (m & ~7); ++k) any |= H[(size_t)k * B + b];
+        if (k < m) {
+#pragma unroll
+            for (int i = 0; i < 7; ++i) any |= k + i < m ? H[(size_t)(k + i) * B + b] : 0u;  // (in flight together)
+        }
         over |= any >= 0x80000000u;
         if (any) mask[b] = 1;
     }
