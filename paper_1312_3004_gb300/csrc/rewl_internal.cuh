@@ -162,6 +162,7 @@ struct SweepPlan {
 
 // Launchers (rewl_kernels.cu).  All enqueue on `s` and return the launch error.
 cudaError_t launch_init(const Model &M, const State &S, cudaStream_t s);
+bool init_by_threads(const Model &M, int num_sms);  // a thread per walker, not a warp
 // kind: SWEEP_REFERENCE / SWEEP_FAST; lanes: 0 = choose from the walker count.
 // A plan with P == 0 means the configuration does not fit (shared memory).
 // lat_mode: where the fast sweep keeps the lattices (0 by size, 1 global, 2 shared).

@@ -108,7 +108,46 @@ __device__ int recount_energy(const uint32_t *w, const Model &M) {
 // that an accepted earlier move touches are carried out together.  (While E < lo
 // a move to E' >= E cannot pass E_hi, since W >= 8.)  q = 10, L = 40, 41 windows
 // of 4: 527 -> 86 us; L = 80, 64 windows of 16: 2675 -> 336 us.
+//
+// Small lattices in great number are a thread's work each: a warp's 32 moves touch
+// one another there, and enough threads hide the chains (init_walkers_kernel).
 constexpr int INIT_THREADS = 64;
+
+// Word i of walker g's drawn configuration.
+template <int BITS>
+__device__ __forceinline__ uint32_t drawn_word(const Model &M, int g, int i) {
+    constexpr int per = 32 / BITS;
+    uint32_t word = 0;
+#pragma unroll
+    for (int c = 0; c < per / 4; ++c) {  // a block of random words is four spins
+        const int s0 = i * per + 4 * c;
+        const uint4 r = philox((uint32_t)(s0 >> 2), 0u, (uint32_t)g, DOM_INIT, M.key0, M.key1);
+        const uint32_t rv[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (s0 + j < M.N) word |= __umulhi(rv[j], (uint32_t)M.q) << ((4 * c + j) * BITS);
+    }
+    return word;
+}
+// The uniform configuration that walker g restarts from, as a word.
+template <int BITS>
+__device__ __forceinline__ uint32_t uniform_word(const Model &M, int g) {
+    const uint32_t c = __umulhi(philox(0u, 0u, (uint32_t)g, DOM_ENTRY, M.key0, M.key1).x, (uint32_t)M.q);
+    return c * (BITS == 8 ? 0x01010101u : 0x11111111u);
+}
+__device__ __forceinline__ unsigned long long entry_moves(const Model &M) {
+    return 1000ull * (unsigned long long)M.N + 1000000ull;  // at most
+}
+// Walker g has entered its window with energy E.
+__device__ __forceinline__ void entered(const Model &M, const State &S, int g, int E) {
+    S.cfg_E[g] = E;
+    S.slot_cfg[g] = (uint32_t)g;
+    // replica g starts in walker g's window
+    const int wg = g / M.m;
+    S.rt_end[g] = M.h < 2 ? 0 : (wg == 0 ? 1 : (wg == M.h - 1 ? 2 : 0));
+    S.rt_trips[g] = 0u;
+    S.t[g] = 0ull;
+}
 
 template <int BITS>
 __global__ void __launch_bounds__(INIT_THREADS) init_kernel(Model M, State S) {
@@ -117,19 +156,7 @@ __global__ void __launch_bounds__(INIT_THREADS) init_kernel(Model M, State S) {
     constexpr unsigned all = 0xffffffffu;
     constexpr int per = 32 / BITS;
     uint32_t *w = S.spins + (size_t)g * M.wpc;
-    for (int i = lane; i < M.wpc; i += 32) {
-        uint32_t word = 0;
-#pragma unroll
-        for (int c = 0; c < per / 4; ++c) {  // a block of random words is four spins
-            const int s0 = i * per + 4 * c;
-            const uint4 r = philox((uint32_t)(s0 >> 2), 0u, (uint32_t)g, DOM_INIT, M.key0, M.key1);
-            const uint32_t rv[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (s0 + j < M.N) word |= __umulhi(rv[j], (uint32_t)M.q) << ((4 * c + j) * BITS);
-        }
-        w[i] = word;
-    }
+    for (int i = lane; i < M.wpc; i += 32) w[i] = drawn_word<BITS>(M, g, i);
     __syncwarp();
     int sat = 0;
     for (int s = lane; s < M.N; s += 32) {
@@ -140,14 +167,12 @@ __global__ void __launch_bounds__(INIT_THREADS) init_kernel(Model M, State S) {
     int E = -__reduce_add_sync(all, sat);
     const int lo = S.e_lo[g / M.m], hi = lo + M.W;
     if (E > hi) {
-        const uint4 r = philox(0u, 0u, (uint32_t)g, DOM_ENTRY, M.key0, M.key1);
-        const uint32_t c = __umulhi(r.x, (uint32_t)M.q);
-        const uint32_t fill = (BITS == 8) ? c * 0x01010101u : c * 0x11111111u;
+        const uint32_t fill = uniform_word<BITS>(M, g);
         for (int j = lane; j < M.wpc; j += 32) w[j] = fill;
         E = -2 * M.N;
     }
     __syncwarp();
-    const unsigned long long max_moves = 1000ull * (unsigned long long)M.N + 1000000ull;
+    const unsigned long long max_moves = entry_moves(M);
     for (unsigned long long n0 = 1; E < lo;) {
         if (n0 > max_moves) {
             if (lane == 0) atomicOr(&S.ctl->error, ERR_ENTRY);
@@ -187,14 +212,40 @@ __global__ void __launch_bounds__(INIT_THREADS) init_kernel(Model M, State S) {
         n0 += (unsigned long long)taken;
         __syncwarp();
     }
-    if (lane != 0) return;
-    S.cfg_E[g] = E;
-    S.slot_cfg[g] = (uint32_t)g;
-    // replica g starts in walker g's window
-    const int wg = g / M.m;
-    S.rt_end[g] = M.h < 2 ? 0 : (wg == 0 ? 1 : (wg == M.h - 1 ? 2 : 0));
-    S.rt_trips[g] = 0u;
-    S.t[g] = 0ull;
+    if (lane == 0) entered(M, S, g, E);
+}
+
+template <int BITS>
+__global__ void __launch_bounds__(INIT_THREADS) init_walkers_kernel(Model M, State S) {
+    const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (g >= M.G) return;
+    uint32_t *w = S.spins + (size_t)g * M.wpc;
+    for (int i = 0; i < M.wpc; ++i) w[i] = drawn_word<BITS>(M, g, i);
+    int E = recount_energy<BITS>(w, M);
+    const int lo = S.e_lo[g / M.m], hi = lo + M.W;
+    if (E > hi) {
+        const uint32_t fill = uniform_word<BITS>(M, g);
+        for (int i = 0; i < M.wpc; ++i) w[i] = fill;
+        E = -2 * M.N;
+    }
+    const unsigned long long max_moves = entry_moves(M);
+    for (unsigned long long n = 1; E < lo; ++n) {
+        if (n > max_moves) {
+            atomicOr(&S.ctl->error, ERR_ENTRY);
+            break;
+        }
+        const uint4 r = philox((uint32_t)n, (uint32_t)(n >> 32), (uint32_t)g, DOM_ENTRY, M.key0, M.key1);
+        const int site = (int)__umulhi(r.x, (uint32_t)M.N);
+        const int cur = spin_get<BITS>(w, site);
+        const int v = (int)__umulhi(r.y, (uint32_t)(M.q - 1));
+        const int nw = v + (v >= cur);
+        const int dE = delta_e<BITS>(w, neighbours(site, M.L, M.N, M.divL), cur, nw);
+        if (dE >= 0) {  // (E < lo: at most E_hi, see above)
+            spin_set<BITS>(w, site, nw);
+            E += dE;
+        }
+    }
+    entered(M, S, g, E);
 }
 
 // ---------------------------------------------------------------------------
@@ -846,7 +897,24 @@ SweepPlan plan_sweep(const Model &M, int num_sms, size_t smem_optin, int kind, i
     return p;
 }
 
+// q = 10, with everything else that a create does, a warp -> a thread per walker: L = 16
+// 32,768 walkers 910 -> 788 us, L = 24 65,536 1611 -> 1092; on the other side of the line
+// L = 16 8192 walkers 667 -> 683, L = 24 8192 708 -> 781, L = 32 32,768 1264 -> 1416.
+bool init_by_threads(const Model &M, int num_sms) {
+    return M.N <= 1024 && (long long)M.G > (long long)num_sms * (20 + M.N / 5);
+}
+
 cudaError_t launch_init(const Model &M, const State &S, cudaStream_t s) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (init_by_threads(M, sms)) {
+        const int grid = (M.G + INIT_THREADS - 1) / INIT_THREADS;
+        if (M.bits == 8) init_walkers_kernel<8><<<grid, INIT_THREADS, 0, s>>>(M, S);
+        else init_walkers_kernel<4><<<grid, INIT_THREADS, 0, s>>>(M, S);
+        return cudaGetLastError();
+    }
     const int grid = (M.G + INIT_THREADS / 32 - 1) / (INIT_THREADS / 32);
     if (M.bits == 8) init_kernel<8><<<grid, INIT_THREADS, 0, s>>>(M, S);
     else init_kernel<4><<<grid, INIT_THREADS, 0, s>>>(M, S);

@@ -60,3 +60,11 @@ def test_narrow_lane_groups_hold_the_walkers_that_an_sm_is_given(tmp_path):
     P = evaluate(tmp_path, ["plan_sweep(model(10, %d, %d, %d, %d, 4), kSms, kShared, SWEEP_FAST, %d).P" % c for c in cases])
     for (L, h, W, m, lanes), p in zip(cases, P):
         assert p >= 0.9 * granted(L, W + 1, -(-h * m // 152), lanes), (L, h, m, lanes, p)
+
+
+def test_entry_form(tmp_path):
+    """(q, L, h, W, m): a thread per walker for many walkers of small lattices"""
+    threads = [(10, 8, 32, 14, 256), (10, 12, 64, 17, 256), (10, 16, 96, 20, 256), (10, 24, 128, 35, 256), (10, 32, 256, 31, 256)]
+    warps = [(2, 8, 4, 73, 2), (10, 16, 32, 58, 256), (10, 24, 32, 131, 256), (10, 32, 128, 62, 256), (10, 64, 512, 63, 256)]
+    rule = ["init_by_threads(model(%d, %d, %d, %d, %d, 4), kSms)" % c for c in threads + warps]
+    assert evaluate(tmp_path, rule) == [1] * len(threads) + [0] * len(warps)
