@@ -344,9 +344,9 @@ rewl_status rewl_batch_create_ext(const rewl_params *jobs, int n, int spin_bits,
 /* Autotuner (no counterpart in the paper: it picks how the batch runs, not
  * what it computes).  Times the batch's candidate configurations -- spin
  * packing 4 or 8 bits (when spin_bits was 0 and every q <= 16), walkers as lane
- * groups of 32 with 36, 72 or 110 KB of shared memory per sweep CTA (when
- * lanes was 0 and the walkers fit) or as a thread each with 32 or 128
- * threads per CTA -- each over `rounds` rounds (after one round that settles
+ * groups of 32 with one walker, two, or two small ones per sweep CTA (as far as
+ * these differ, when lanes was 0 and the walkers fit) or as a thread each with 32
+ * or 128 threads per CTA -- each over `rounds` rounds (after one round that settles
  * it), by CUDA events on the batch's stream and the WL proposals counted, and
  * leaves the batch in the fastest one.  The rounds it runs are ordinary rounds
  * of every instance (no configuration changes a result).  The choice is
@@ -358,7 +358,7 @@ rewl_status rewl_batch_create_ext(const rewl_params *jobs, int n, int spin_bits,
 typedef struct rewl_tune_entry {
     int spin_bits;      /* 4 or 8 */
     int lanes;          /* 32 (lane groups) or 1 (a thread per walker) */
-    int cta_kb;         /* lane groups: shared memory per sweep CTA (KB), else 0 */
+    int cta_kb;         /* lane groups: shared memory of the largest sweep CTA (KB), else 0 */
     int threads;        /* a thread per walker: threads per CTA, else 0 */
     double flips_per_s; /* WL proposals per second measured */
 } rewl_tune_entry;

@@ -24,11 +24,12 @@ namespace {
 
 constexpr int kBatchGraphRounds = 4;
 constexpr int kSideStreams = 7;
-// Walkers of a sweep CTA in lane groups: a quarter of what fits its shared memory
-// (and the most a CTA can hold).  A CTA ends with its slowest walker, and small
-// CTAs fill an SM's shared memory: 64 instances (1775 walkers) 1.42 -> 1.36 ms a
-// round, 512 instances 6.9 -> 5.7 ms.
-constexpr int kCtaShare = 4;
+// Walkers of a sweep CTA in lane groups: two where both fit this many KB, else one.
+// A CTA ends with its slowest walker, and small CTAs fill an SM's shared memory:
+// up to eight walkers in 72 KB -> this, 64 instances (1775 walkers) 1.42 -> 1.36 ms
+// a round, 512 instances 6.9 -> 5.7 ms.
+constexpr int kPairKb = 18, kPairAlways = 1 << 20, kPairNever = 0;
+int walkers_per_cta(size_t stride, int pair_kb) { return 2 * stride <= (size_t)pair_kb * 1024 ? 2 : 1; }
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -43,7 +44,7 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 struct Config {
     int bits = 8;           // spins per configuration word: 4 or 8 bits each
     int lanes = 32;         // 32: lane groups, state staged in shared memory; 1: a thread per walker
-    int cta_kb = 72;        // lanes 32: shared memory per sweep CTA (walkers per CTA follow)
+    int pair_kb = kPairKb;  // lanes 32: walkers_per_cta
     int threads = 32;       // lanes 1: threads per CTA (a warp: 1775 of them spread evenly over 152 SMs)
 };
 
@@ -240,7 +241,6 @@ rewl_status configure(rewl_batch_s *b, const Config &c) {
         for (int w = 0; w < b->inst[(size_t)i]->M.h; ++w) wins.push_back({i, w});
     b->n_wins = (int)wins.size();
     b->classes.clear();
-    const size_t budget = (size_t)c.cta_kb * 1024;
     for (int i = 0; i < n; ++i) {
         rewl_s *h = b->inst[(size_t)i];
         tab[(size_t)i].M = h->M;
@@ -267,8 +267,8 @@ rewl_status configure(rewl_batch_s *b, const Config &c) {
             for (int g = 0; g < h->M.G; ++g) sc.walkers.push_back({i, g});
             continue;
         }
-        int P = (int)(std::max(budget, (size_t)lay.stride) / (size_t)lay.stride);
-        P = std::max(1, std::min(P, 256 / sc.lanes) / kCtaShare);
+        int P = walkers_per_cta((size_t)lay.stride, c.pair_kb);
+        if ((size_t)P * (size_t)lay.stride > (size_t)h->smem_optin) P = 1;
         for (int g0 = 0; g0 < h->M.G; g0 += P) sc.items.push_back({i, g0, std::min(P, h->M.G - g0), 0});
         sc.smem = std::max(sc.smem, (size_t)P * (size_t)lay.stride);
         sc.threads = std::max(sc.threads, P * sc.lanes);
@@ -323,6 +323,13 @@ rewl_status configure(rewl_batch_s *b, const Config &c) {
     if (e != cudaSuccess) return fail(REWL_ERR_CUDA, "batch configuration: %s", cudaGetErrorString(e));
     b->cfg = c;
     return build_batch_graph(b);
+}
+
+// Shared memory of the largest sweep CTA in KB, rounded up (0: a thread per walker).
+int cta_kb(const rewl_batch_s *b) {
+    size_t most = 0;
+    for (const SweepClass &c : b->classes) most = std::max(most, c.smem);
+    return (int)((most + 1023) / 1024);
 }
 
 }  // namespace
@@ -464,8 +471,19 @@ rewl_status rewl_batch_autotune(rewl_batch_t b, int rounds, rewl_tune_entry *ent
             c.bits = bits;
             c.lanes = lanes;
             if (lanes == 32) {
-                for (int kb : {36, 72, 110}) {
-                    c.cta_kb = kb;
+                // (no two that give every instance the same)
+                std::vector<std::vector<int>> seen;
+                for (int kb : {kPairKb, kPairNever, kPairAlways}) {
+                    std::vector<int> P;
+                    for (rewl_s *h : b->inst) {
+                        rewl::Model M = h->M;
+                        M.bits = bits;
+                        M.wpc = (M.N * bits + 31) / 32;
+                        P.push_back(walkers_per_cta((size_t)rewl::fast_layout(M, 32).stride, kb));
+                    }
+                    if (std::find(seen.begin(), seen.end(), P) != seen.end()) continue;
+                    seen.push_back(P);
+                    c.pair_kb = kb;
                     cands.push_back(c);
                 }
             } else {
@@ -505,7 +523,7 @@ rewl_status rewl_batch_autotune(rewl_batch_t b, int rounds, rewl_tune_entry *ent
             rewl_tune_entry &en = entries[n_done];
             en.spin_bits = cands[i].bits;
             en.lanes = cands[i].lanes;
-            en.cta_kb = cands[i].lanes == 32 ? cands[i].cta_kb : 0;
+            en.cta_kb = cta_kb(b);
             en.threads = cands[i].lanes == 1 ? cands[i].threads : 0;
             en.flips_per_s = rate;
         }
@@ -534,7 +552,7 @@ rewl_status rewl_batch_config(rewl_batch_t b, int *spin_bits, int *lanes, int *c
     if (!b) return fail(REWL_ERR_ARG, "NULL batch");
     if (spin_bits) *spin_bits = b->cfg.bits;
     if (lanes) *lanes = b->cfg.lanes;
-    if (cta_kb) *cta_kb = b->cfg.lanes == 32 ? b->cfg.cta_kb : 0;
+    if (cta_kb) *cta_kb = ::cta_kb(b);
     if (threads) *threads = b->cfg.lanes == 1 ? b->cfg.threads : 0;
     return REWL_OK;
     REWL_API_CATCH

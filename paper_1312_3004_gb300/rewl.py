@@ -264,7 +264,7 @@ class Batch:
         return [{k: getattr(ent[i], k) for k, _ in _lib.TuneEntry._fields_} for i in range(n.value)], bool(cached.value)
 
     def config(self):
-        """The batch's configuration: spin bits, lanes, CTA shared memory (KB) or threads per CTA."""
+        """The batch's configuration: spin bits, lanes, shared memory of the largest sweep CTA (KB) or threads per CTA."""
         v = [C.c_int(0) for _ in range(4)]
         check(self._L.rewl_batch_config(self._h, *[C.byref(x) for x in v]))
         return dict(zip(("spin_bits", "lanes", "cta_kb", "threads"), (x.value for x in v)))
