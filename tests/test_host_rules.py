@@ -68,3 +68,12 @@ def test_entry_form(tmp_path):
     warps = [(2, 8, 4, 73, 2), (10, 16, 32, 58, 256), (10, 24, 32, 131, 256), (10, 32, 128, 62, 256), (10, 64, 512, 63, 256)]
     rule = ["init_by_threads(model(%d, %d, %d, %d, %d, 4), kSms)" % c for c in threads + warps]
     assert evaluate(tmp_path, rule) == [1] * len(threads) + [0] * len(warps)
+
+
+def test_conflict_marks_of_wide_windows(tmp_path):
+    """512 where ln g shadow and lattice pass 96 KB; else one per site, 8192, or 2048
+    beside a lattice in global memory"""
+    cases = [(80, 1, 12800, 0, 512), (200, 20, 13914, 1, 512), (78, 1, 12168, 0, 512), (91, 5, 8281, 0, 8192),
+             (80, 64, 766, 0, 6400), (200, 40, 7442, 1, 2048)]
+    marks = evaluate(tmp_path, ["fast_layout(model(10, %d, %d, %d, 1, 4), 32, %d).marks" % c[:4] for c in cases])
+    assert marks == [c[4] for c in cases]
