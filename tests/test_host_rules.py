@@ -20,7 +20,7 @@ def test_faulting_in_a_result_buffer_keeps_what_it_holds(tmp_path):
     """a read that fails later leaves the caller's buffer as it was; every page is
     looked at once, whatever the alignment"""
     assert evaluate(tmp_path, [r"""([] {
-        std::vector<unsigned char> v(1000003);
+        std::vector<unsigned char> v(9000003);
         for (size_t i = 0; i < v.size(); ++i) v[i] = (unsigned char)(i * 7 + 1);
         rewl::host::fault_in(v.data() + 1, v.size() - 1);
         rewl::host::fault_in(v.data(), 0);
