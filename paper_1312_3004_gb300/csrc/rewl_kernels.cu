@@ -853,12 +853,16 @@ SweepPlan plan_sweep(const Model &M, int num_sms, size_t smem_optin, int kind, i
     if (kind == SWEEP_FAST) {
         // lane groups while walkers are few (each walker's chain is what bounds
         // the rate); a thread per walker, state in global memory, once there are
-        // enough of them to fill the SMs by themselves (measured crossover on
-        // GB300: between 4096 and 16384 walkers)
+        // enough of them to fill the SMs by themselves.  Rounds of 2000 steps at
+        // ln f = 2^-20, lane groups / threads, in us: q = 10, L = 80, 64 windows: 53
+        // walkers per SM 756 / 1306, 80 1122 / 1472, 107 1530 / 1630; L = 16: 53 516 /
+        // 901, 80 692 / 866, 107 922 / 935; L = 40: 80 679 / 983, 107 922 / 1194
+        // (L = 160, staged at 33 KB a walker, crosses earlier: 26 1437 / 2228, 53 2886 /
+        // 3033, 80 4352 / 3543)
         // (lane groups are 32 lanes at every lattice size: a batch of 32 takes about
-        // as long as one of 8, also where the proposals of a batch touch each other
-        // -- L = 8 Ising, 8 walkers: 615 us a round of 10^4 steps against 1346 with
-        // 8 lanes and 934 with 16; q = 10, L = 20: 708 against 1415 and 1095)
+        // as long as one of 8, also where the proposals of a batch touch each other;
+        // rounds of 2000 steps at ln f = 1, 32 / 16 / 8 lanes, in us: L = 8 Ising, 8
+        // walkers 183 / 307 / 392; q = 10, L = 20, 32 walkers 166 / 265 / 329)
         const bool chosen = lanes <= 0;
         if (chosen) lanes = M.G <= 80 * num_sms ? 32 : 1;
         // a window too wide for a lane group's shared memory (its ln g shadow):

@@ -1,6 +1,6 @@
 // rewl_probe.cu -- rewl_measure_pipes: issue rates of the pipes the WL step
 // uses, measured on the current device, for the per-flip roofline of the
-// benchmark (the measured peaks file has HBM and bf16 figures only).
+// benchmark (published peaks cover HBM and the tensor types only).
 //
 // Throughput: one CTA of 1024 threads per SM (its dynamic shared memory keeps
 // a second CTA off the SM), each thread running 8 independent chains of one
